@@ -56,9 +56,16 @@ int reg_tile_qubits(int dtype) { return (dtype == LQS_C64 ? 4 : 3) + kRegThreadB
 
 // Register bits per thread of a compiled forward segment.  The tile keeps its
 // reg_tile_qubits; fewer register bits give more threads per tile (2^(k - r)).
+// A compiled segment keeps one 64 KiB buffer per tile, so two CTAs share an SM
+// and one computes while the other exchanges, waits for a tile or stores; both
+// together hold 16 (4 register bits, 128 registers) or 32 (3 bits, 64
+// registers) warps.  Measured, 30-qubit 10-layer ansatz / 29-qubit QFT / 24-qubit
+// universal circuit, complex128: one CTA per SM with three buffers 525 / 35.2 /
+// 7.57 ms; two CTAs with 3 register bits 450 / 32.2 / 6.53 ms, with 4 (a
+// quarter fewer exchanges) 444 / 31.6 / 6.29 ms.
 // The interpreter keeps RegR's count.
 #ifndef LQS_SEG_RBITS_C128
-#define LQS_SEG_RBITS_C128 3
+#define LQS_SEG_RBITS_C128 4
 #endif
 template <class A> struct JitR { static constexpr int r = LQS_SEG_RBITS_C128; };
 template <> struct JitR<ArF32> { static constexpr int r = 4; };

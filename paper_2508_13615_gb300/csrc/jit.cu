@@ -187,10 +187,7 @@ class SegGen {
   // gradient partials (seg_scales) and folds into a diagonal run or a final
   // scale; launches whose product of m00's is too small run elsewhere.
   bool unit_adj() const { return adj_ && aname_ == std::string("lqs::ArDF"); }
-  // Complex64 forward segments do too little arithmetic per tile to hide a
-  // tile load behind it: they keep two incoming buffers (two tiles in flight
-  // per CTA) and run every layout exchange through one buffer.
-  bool deep() const { return !adj_ && aname_ == std::string("lqs::ArF32"); }
+  int npf_ = 0;  // forward: places where the next tile's load could start (after each exchange)
   void flush_pending(bool all);
   // runs f once per state, with V() naming that state's variables
   template <class F>
@@ -509,11 +506,13 @@ bool SegGen::exchange_safe(int buf, const std::vector<uint8_t>& wown) const {
 }
 
 void SegGen::emit_layout(const TOp& t) {
-  // Each state is written in the current layout and read back in the new one
-  // through its own buffer.  The buffers alternate, so one barrier per state
-  // suffices: the previous reader of a buffer finished before the
-  // intervening exchange's barrier (or the barriers at the top of the tile
-  // loop).  A folded permutation run (t.fold) moves every amplitude from its
+  // Each state is written in the current layout and read back in the new one.
+  // Forward programs use the tile's one buffer; the ordering check below adds a
+  // block barrier before the writes when the previous exchange's readers are
+  // not ordered before them.  Adjoint programs alternate between two buffers
+  // (pairs), so one barrier per exchange suffices: the previous reader of a
+  // buffer finished before the intervening exchange's barrier (or the barriers
+  // at the top of the tile loop).  A folded permutation run (t.fold) moves every amplitude from its
   // storage position x to F x ^ c on the way: the writes go to the permuted
   // positions, the reads are those of the new layout.
   const TFold* F = t.fold && folds_ ? &folds_[t.fold - 1] : nullptr;
@@ -622,7 +621,7 @@ void SegGen::emit_layout(const TOp& t) {
   each([&]() {
     const int xi = xb_;
     const char* X = xb_ ? "XB" : "XA";
-    if (!deep()) xb_ ^= 1;  // deep: XA only (the second incoming buffer took XB's place)
+    if (adj_) xb_ ^= 1;  // forward: the tile's one buffer
     std::copy(saved_slot, saved_slot + 4, slot_);  // barrier groups compare with the current layout
     std::copy(saved_thr, saved_thr + 16, thr_);
     bool unsafe = !exchange_safe(xi, wown);
@@ -660,6 +659,7 @@ void SegGen::emit_layout(const TOp& t) {
       o_ << "      " << pfx_ << e << " = lqs::ld_w(&" << X << "[" << xacc(xs, je(e)) << "]);\n";
     o_ << "    }\n";
   });
+  if (!adj_) o_ << "@PF" << ++npf_ << "@";
   for (int e = 0; e < R_; ++e) vm_[e] = e;
   if (t.e0 != t.ecmask) {  // relabelling SWAPs: from here on amplitudes carry their logical positions
     set_layout(t.e0);
@@ -843,7 +843,7 @@ bool SegGen::emit_grad_block(const TOp* ops, int count) {
     auto it = sums.find(key);
     if (it == sums.end()) {
       const std::string sn = fresh("s");
-      o_ << "      lqs::jit::GAcc<A>::T " << sn << " = lqs::jit::GAcc<A>::zero();\n";
+      o_ << "      lqs::jit::GAcc<A>::B " << sn << " = lqs::jit::GAcc<A>::bzero();\n";
       for (int e = 0; e < R_; ++e)
         if (((uint32_t)e & regc) == regc)
           o_ << "      lqs::jit::wadd(" << sn << ", " << wn << "_" << e << ", " << ((sm >= 0 && ((e >> sm) & 1)) ? "true" : "false")
@@ -853,7 +853,7 @@ bool SegGen::emit_grad_block(const TOp* ops, int count) {
     const std::string slot = "wacc + warp * " + std::to_string(kMaxGradSlotsJit) + " + " + std::to_string(t.gslot);
     if (thc) {  // a per-lane predicate: this partial needs its own warp sum
       std::string val = rs.empty() ? it->second : "lqs::jit::gneg(" + it->second + ", " + rs + ")";
-      val = "(" + p + " && " + tp + ") ? " + val + " : lqs::jit::GAcc<A>::zero()";
+      val = "(" + p + " && " + tp + ") ? " + val + " : lqs::jit::GAcc<A>::bzero()";
       if (lbit >= 0) val = "lqs::jit::gneg(" + val + ", ((tid >> " + std::to_string(lbit) + ") & 1u) != 0u)";
       o_ << "      lqs::jit::gflush(" << val << ", " << slot << ");  // gradient slot " << t.gslot << "\n";
       continue;
@@ -1214,6 +1214,13 @@ bool SegGen::emit_op(const TOp& t) {
   }
 }
 
+// Forward segments run two CTAs per SM, each with one tile buffer: bulk loads
+// land in it, and once the tile is in registers the layout exchanges go
+// through it.  After the last exchange has been read the buffer is free and
+// the next tile's load starts, behind the remaining ops and the stores of this
+// tile and the whole work of the other CTA.  FP32 pipe busy 57-68% against
+// 52-56% with one CTA per SM and a prefetch buffer (24-qubit ansatz); adjoint
+// sweeps hold two states and keep one CTA with separate exchange buffers.
 const char* kSkeletonHead = R"(
 extern "C" __global__ void __launch_bounds__(@NTH@, @MINB@)
 @NAME@(A::S* __restrict__ psi, @LAMP@const __grid_constant__ SegArgs P, @PARTP@int* status@FMTP@) {
@@ -1224,7 +1231,7 @@ extern "C" __global__ void __launch_bounds__(@NTH@, @MINB@)
   const lqs::TileGeom& G = P.g;
   S* S0 = reinterpret_cast<S*>(smem_raw);  // incoming tiles (bulk loads, prefetched one tile ahead)
   S* S0L = S0 + @NT@;                      // incoming lambda tiles (adjoint only)
-  W* XA = reinterpret_cast<W*>(S0 + @NT@ * @NIN@);  // layout exchanges alternate between XA and XB
+  W* XA = reinterpret_cast<W*>(S0 + @NT@ * @NIN@);  // layout exchanges (forward: in the tile's own buffer)
   W* XB = XA + @NT@;
   W* XC = XB + @NT@;  // complex128 adjoint: the second pair of exchange buffers
   W* XD = XC + @NT@;
@@ -1257,57 +1264,6 @@ extern "C" __global__ void __launch_bounds__(@NTH@, @MINB@)
     if (!ok) break;
     // the next phase's byte count goes up before any of its copies is issued
     if (tid == 0 && t + gridDim.x < G.ntiles) lqs::jit::seg_expect(G, bar, @NSTATES@);
-)";
-
-// Complex64 forward segments: two incoming buffers and two barriers; tile
-// it of this CTA lands in buffer it & 1 (barrier phase (it >> 1) & 1).
-const char* kSkeletonHeadDeep = R"(
-extern "C" __global__ void __launch_bounds__(@NTH@, @MINB@)
-@NAME@(A::S* __restrict__ psi, const __grid_constant__ SegArgs P, int* status, const unsigned fmt) {
-  typedef A::S S;
-  typedef A::W W;
-  typedef A::C C;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const lqs::TileGeom& G = P.g;
-  S* S0 = reinterpret_cast<S*>(smem_raw);      // incoming tiles, two buffers (two tiles in flight)
-  W* XA = reinterpret_cast<W*>(S0 + @NT@ * 2u);  // every layout exchange
-  W* XB = XA;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(XA + @NT@);
-  const uint32_t tid = threadIdx.x;
-  (void)XB;
-  (void)fmt;
-  uint64_t t = blockIdx.x;
-  const uint64_t grid = gridDim.x;
-  if (tid == 0) {
-    lqs::mbar_init(bar, 1);
-    lqs::mbar_init(bar + 1, 1);
-    lqs::fence_mbar_init();
-    if (t < G.ntiles) lqs::jit::seg_expect(G, bar, 1u);
-    if (t + grid < G.ntiles) lqs::jit::seg_expect(G, bar + 1, 1u);
-  }
-  __syncthreads();
-  const uint64_t my_roff = tid < (1u << G.r) ? lqs::row_offset(G, tid) : 0ull;
-  if (t < G.ntiles) lqs::jit::seg_copy(G, S0, psi, lqs::tile_base(G, t), bar, my_roff);
-  if (t + grid < G.ntiles) lqs::jit::seg_copy(G, S0 + @NT@, psi, lqs::tile_base(G, t + grid), bar + 1, my_roff);
-  uint32_t it = 0;
-  bool ok = true;
-@TBL@@PRE@  for (; t < G.ntiles; t += grid, ++it) {
-    const uint64_t base = lqs::tile_base(G, t);
-    S* SIN = S0 + @NT@ * (it & 1u);
-    uint64_t* BAR = bar + (it & 1u);
-    ok = __syncthreads_and(lqs::mbar_wait(BAR, (it >> 1) & 1u));
-    if (!ok) break;
-    // the byte count of this buffer's next tile goes up before its copies are issued
-    if (tid == 0 && t + 2ull * grid < G.ntiles) lqs::jit::seg_expect(G, BAR, 1u);
-)";
-
-const char* kSkeletonTailDeep = R"(  }
-  if (!ok && tid == 0) {
-    lqs::flag_timeout(status, 4);
-    lqs::mbar_wait(bar + (it & 1u), (it >> 1) & 1u);  // let the copies in flight land (bounded)
-    if (t + grid < G.ntiles) lqs::mbar_wait(bar + ((it + 1u) & 1u), ((it + 1u) >> 1) & 1u);
-  }
-}
 )";
 
 const char* kSkeletonTail = R"(  }
@@ -1378,7 +1334,7 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
     o_ << "    W";
     for (int e = 0; e < R_; ++e) o_ << (e ? ", " : " ") << pfx_ << e;
     o_ << ";\n";
-    const char* sin = pfx_[0] == 'v' ? (deep() ? "SIN" : "S0") : "S0L";
+    const char* sin = pfx_[0] == 'v' ? "S0" : "S0L";
     if (split_io()) {  // the previous segment of this call left hi/lo pairs
       o_ << "    if (fmt & 1u) {\n";
       for (int e = 0; e < R_; ++e)
@@ -1395,18 +1351,15 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
     set_layout(logical);
     o_ << "    jt = " << jt_expr() << ";\n";
   }
-  if (deep())
-    o_ << "    __syncthreads();  // this incoming buffer is free: the tile two ahead goes into it\n"
-          "    { const uint64_t tn = t + 2ull * gridDim.x;\n"
-          "      if (tn < G.ntiles) {\n"
-          "        lqs::jit::seg_copy(G, SIN, psi, lqs::tile_base(G, tn), BAR, my_roff);\n";
-  else
+  if (adj_) {
     o_ << "    __syncthreads();  // the incoming buffers are free: prefetch the next tile into them\n"
           "    { const uint64_t tn = t + gridDim.x;\n"
           "      if (tn < G.ntiles) {\n"
-          "        lqs::jit::seg_copy(G, S0, psi, lqs::tile_base(G, tn), bar, my_roff);\n";
-  if (adj_) o_ << "        lqs::jit::seg_copy(G, S0L, lam, lqs::tile_base(G, tn), bar, my_roff);\n";
-  o_ << "      } }\n";
+          "        lqs::jit::seg_copy(G, S0, psi, lqs::tile_base(G, tn), bar, my_roff);\n"
+          "        lqs::jit::seg_copy(G, S0L, lam, lqs::tile_base(G, tn), bar, my_roff);\n      } }\n";
+  } else {
+    o_ << "    __syncthreads();  // the tile has been read: its buffer serves the exchanges\n@PF0@";
+  }
   for (int i = first; i < nops; ++i) {
     if (ops[i].kind == K_LAYOUT) {
       if (i == nops - 1 && !ops[i].fold) {
@@ -1478,14 +1431,20 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
       os << ind << "}\n";
     };
     o_ << "    { const uint64_t tno = t + gridDim.x;\n";
-    fill(o_, "tno", deep() ? "((it + 1u) & 1u) * " + nof : "phase * " + nof, "      ");
+    fill(o_, "tno", "phase * " + nof, "      ");
     o_ << "    }\n";
     pre_ << "  __syncthreads();\n";
     fill(pre_, "t", "0u", "  ");
   }
-  std::string body = replace_all(o_.str(), "@OFCUR@",
-                                 (deep() ? std::string("(it & 1u) * ") : std::string("(phase ^ 1u) * ")) +
-                                     std::to_string(ofac_.size()) + "u");
+  std::string body = replace_all(o_.str(), "@OFCUR@", "(phase ^ 1u) * " + std::to_string(ofac_.size()) + "u");
+  if (!adj_) {
+    // the next tile's load starts once the last exchange has been read
+    for (int i = 0; i < npf_; ++i) body = replace_all(body, "@PF" + std::to_string(i) + "@", "");
+    body = replace_all(body, "@PF" + std::to_string(npf_) + "@",
+                       std::string(npf_ ? "    lqs::fence_proxy_async();\n    __syncthreads();  // the buffer is free\n" : "") +
+                           "    { const uint64_t tn = t + gridDim.x;\n"
+                           "      if (tn < G.ntiles) lqs::jit::seg_copy(G, S0, psi, lqs::tile_base(G, tn), bar, my_roff); }\n");
+  }
   const uint64_t h = fnv1a(body) ^ (fnv1a(pre_.str()) * 31u) ^ ((uint64_t)ncoef << 48) ^ ((uint64_t)k_ << 40) ^
                      ((uint64_t)b_ << 36) ^ ((uint64_t)ngrad << 24) ^ (adj_ ? 0x5a5aull : 0ull) ^ fnv1a(aname_);
   char nm[40];
@@ -1498,23 +1457,23 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
     << "typedef unsigned char uint8_t;\ntypedef signed char int8_t;\ntypedef short int16_t;\ntypedef unsigned short uint16_t;\n"
        "typedef unsigned int uint32_t;\ntypedef unsigned long long uint64_t;\n"
     << "#include \"tile.cuh\"\n#include \"jit_dev.cuh\"\n"
-    << "typedef " << aname_ << " A;\n"
+    << "typedef " << jit_policy(aname_) << " A;\n"
     << "struct SegArgs {\n  lqs::TileGeom g;\n  A::C coef[" << std::max(ncoef, 1) << "];\n";
   if (nu_) s << "  A::C gscale;\n  uint32_t usel[" << (nu_ + 31) / 32 << "];\n";
   s << "};\n";
-  std::string head = replace_all(deep() ? kSkeletonHeadDeep : kSkeletonHead, "@NAME@", kname);
+  std::string head = replace_all(kSkeletonHead, "@NAME@", kname);
   head = replace_all(head, "@NTH@", std::to_string(nth));
-  // resident CTAs per SM the register budget aims at: forward 512 threads
-  // per SM; adjoint 3 x 128, with 256 threads 2 (4 amplitudes of each state
+  // resident CTAs per SM the register budget aims at: forward two (1024 threads
+  // per SM with 128 bytes of state per thread, 512 with 256); adjoint 3 x 128, with 256 threads 2 (4 amplitudes of each state
   // per thread) or 1 (8 or more), with 512 threads 1
-  const int minb = !adj_ ? std::max(1, 512 / nth) : nth <= 128 ? 3 : nth >= 512 ? 1 : (R_ * sz_ <= 64 ? 2 : 1);
+  const int minb = !adj_ ? std::max(1, (R_ * sz_ <= 128 ? 1024 : 512) / nth) : nth <= 128 ? 3 : nth >= 512 ? 1 : (R_ * sz_ <= 64 ? 2 : 1);
   head = replace_all(head, "@MINB@", std::to_string(minb));
   head = replace_all(head, "@LAMP@", adj_ ? "A::S* __restrict__ lam, " : "");
   head = replace_all(head, "@PARTP@", adj_ ? "double* partial, " : "");
   head = replace_all(head, "@FMTP@", ", const unsigned fmt");
   head = replace_all(head, "@NT@", std::to_string(1u << k_) + "u");
-  head = replace_all(head, "@NIN@", adj_ ? "2u" : "1u");
-  head = replace_all(head, "@NX@", xpair_ ? "4u" : "2u");
+  head = replace_all(head, "@NIN@", adj_ ? "2u" : "0u");
+  head = replace_all(head, "@NX@", xpair_ ? "4u" : adj_ ? "2u" : "1u");
   head = replace_all(head, "@NSTATES@", adj_ ? "2u" : "1u");
   head = replace_all(head, "@NWACC@", std::to_string(adj_ ? nwarps * kMaxGradSlotsJit : 0) + "u");
   head = replace_all(head, "@LAMCOPY0@",
@@ -1524,7 +1483,7 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
                          (nut_ ? "  __shared__ C UT[" + std::to_string(nut_) + "];\n" : std::string()) +
                          (ofac_.empty() ? std::string() : "  __shared__ C OF[" + std::to_string(2 * ofac_.size()) + "];\n"));
   head = replace_all(head, "@PRE@", pre_.str());
-  std::string tail = deep() ? kSkeletonTailDeep : kSkeletonTail;
+  std::string tail = kSkeletonTail;
   std::string gout;
   if (adj_) {
     gout = replace_all(kGradOut, "@NGRAD@", std::to_string(ngrad));
@@ -2044,10 +2003,7 @@ int jit_launch(const TileProg<A>& P, int r, SV* sv, double bytes, double flops, 
   Entry* e = entry_for(P, r, false, false, nullptr);
   const int dev = sv->device;
   const int threads = 1 << (P.g.k - r);
-  // incoming tile and two exchange buffers, or (complex64) two incoming
-  // tiles and one exchange buffer; one or two barriers
-  const bool deep = std::is_same<A, ArF32>::value;
-  const size_t smem = 3 * ((size_t)sizeof(typename A::S) << P.g.k) + (deep ? 32 : 16);
+  const size_t smem = ((size_t)sizeof(typename A::S) << P.g.k) + 16;  // the tile and its barrier
   CUfunction fn;
   int per_sm;
   LQS_TRY(entry_function(e, dev, smem, threads, &fn, &per_sm));

@@ -9,6 +9,12 @@
 
 namespace lqs {
 
+// The arithmetic policy a compiled kernel of policy `aname` runs on: packed
+// double-float for ArDF (jit_dev.cuh), the policy itself otherwise.
+inline std::string jit_policy(const std::string& aname) {
+  return aname == "lqs::ArDF" ? "lqs::jit::ArDFP" : aname;
+}
+
 int jit_mode();
 // Whether compiled segments may run for an n-qubit state under the current mode.
 bool jit_enabled_for(int n);

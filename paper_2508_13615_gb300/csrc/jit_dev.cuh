@@ -60,96 +60,169 @@ template <class A> struct Lz {
     return r;
   }
 };
-template <> struct Lz<ArDF> {
-  using W = DFC;
+// Double-float amplitudes of compiled segments, two floats to a register pair
+// (arith.cuh f2): the leading parts of (re, im) and their low parts.  Every
+// operation runs on both components at once, in the order and with the
+// roundings of the scalar forms (arith.cuh df_prod, df_mac), so results are
+// those of ArDF bit for bit.
+struct P2 { f2 h, l; };   // two double-floats
+struct PAcc { f2 s, e; };  // two accumulators (leading sums, collected errors)
+__device__ __forceinline__ P2 p2_raw(const PAcc& a) { return P2{a.s, a.e}; }
+__device__ __forceinline__ P2 p2_neg(const P2& a) { return P2{f2_neg(a.h), f2_neg(a.l)}; }
+__device__ __forceinline__ P2 p2_swap(const P2& a) { return P2{f2_swap(a.h), f2_swap(a.l)}; }
+__device__ __forceinline__ P2 p2_norm(const PAcc& a) {
+  const f2 h = f2_add(a.s, a.e);
+  return P2{h, f2_sub(a.e, f2_sub(h, a.s))};
+}
+__device__ __forceinline__ PAcc p2_prod(const P2& a, const P2& c) {
+  const f2 p = f2_mul(a.h, c.h);
+  f2 e = f2_fma(a.h, c.h, f2_neg(p));
+  e = f2_fma(a.h, c.l, e);
+  e = f2_fma(a.l, c.h, e);
+  return PAcc{p, e};
+}
+__device__ __forceinline__ void p2_acc(PAcc& A, f2 x, f2 xe) {  // A += x + xe, TwoSum on the leading parts
+  const f2 s = f2_add(A.s, x);
+  const f2 bp = f2_sub(s, A.s);
+  const f2 err = f2_add(f2_sub(A.s, f2_sub(s, bp)), f2_sub(x, bp));
+  A.s = s;
+  A.e = f2_add(A.e, f2_add(err, xe));
+}
+__device__ __forceinline__ void p2_mac(PAcc& A, const P2& a, const P2& c) {
+  const PAcc q = p2_prod(a, c);
+  p2_acc(A, q.s, q.e);
+}
+// lane 0 / lane 1 as scalar double-floats
+__device__ __forceinline__ void p2_lanes(const P2& a, DF& x, DF& y) {
+  f2_unpack(a.h, x.h, y.h);
+  f2_unpack(a.l, x.l, y.l);
+}
+}  // namespace jit
+
+// 128-bit shared-memory and global accesses of working amplitudes.
+__device__ __forceinline__ void st_w(jit::P2* p, const jit::P2& v) {
+  *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v.h, v.l);
+}
+__device__ __forceinline__ jit::P2 ld_w(const jit::P2* p) {
+  const ulonglong2 f = *reinterpret_cast<const ulonglong2*>(p);
+  return jit::P2{f.x, f.y};
+}
+
+namespace jit {
+// A real coefficient; nh = -h, so that a product's error term needs no
+// negation of the product.
+struct R2 { f2 h, nh, l; };
+
+// The policy of compiled complex128 double-float segments: ArDF's storage and
+// coefficients, packed working amplitudes.
+struct ArDFP {
+  using S = double2;
+  using W = P2;
   using C = DFK;
-  static __device__ __forceinline__ DF raw(const DAcc& a) { return DF{a.s, a.e}; }
-  static __device__ __forceinline__ W cmul(const C& c, const W& a) {
-    DAcc re = df_prod(a.re, c.re);
-    df_mac(re, df_neg(a.im), c.im);
-    DAcc im = df_prod(a.im, c.re);
-    df_mac(im, a.re, c.im);
-    return W{raw(re), raw(im)};
+  using R = R2;
+  static __device__ __forceinline__ W load(const S& s) {
+    const DF re = d2df(s.x), im = d2df(s.y);
+    return W{f2_pack(re.h, im.h), f2_pack(re.l, im.l)};
   }
-  static __device__ __forceinline__ W cmac2(const C& c0, const W& a, const C& c1, const W& b) {
-    DAcc re = df_prod(a.re, c0.re);
-    df_mac(re, df_neg(a.im), c0.im);
-    df_mac(re, b.re, c1.re);
-    df_mac(re, df_neg(b.im), c1.im);
-    DAcc im = df_prod(a.im, c0.re);
-    df_mac(im, a.re, c0.im);
-    df_mac(im, b.im, c1.re);
-    df_mac(im, b.re, c1.im);
-    return W{raw(re), raw(im)};
+  static __device__ __forceinline__ S store(const W& w) {
+    DF re, im;
+    p2_lanes(w, re, im);
+    return make_double2(df2d(re), df2d(im));
   }
-  static __device__ __forceinline__ W cmac4(const C* c, const W* a) {
-    DAcc re = df_prod(a[0].re, c[0].re);
-    df_mac(re, df_neg(a[0].im), c[0].im);
-    DAcc im = df_prod(a[0].im, c[0].re);
-    df_mac(im, a[0].re, c[0].im);
-#pragma unroll
-    for (int k = 1; k < 4; ++k) {
-      df_mac(re, a[k].re, c[k].re);
-      df_mac(re, df_neg(a[k].im), c[k].im);
-      df_mac(im, a[k].im, c[k].re);
-      df_mac(im, a[k].re, c[k].im);
-    }
-    return W{raw(re), raw(im)};
-  }
-  static __device__ __forceinline__ W rmac2(const DF& c0, const W& a, const DF& c1, const W& b) {
-    DAcc re = df_prod(a.re, c0);
-    df_mac(re, b.re, c1);
-    DAcc im = df_prod(a.im, c0);
-    df_mac(im, b.im, c1);
-    return W{raw(re), raw(im)};
-  }
-  static __device__ __forceinline__ C kmul(const C& a, const C& b) {
-    const W r = cmul(a, W{b.re, b.im});
-    return C{r.re, r.im};
-  }
-  static __device__ __forceinline__ void renorm(W& w) {
-    w.re = df_norm(DAcc{w.re.h, w.re.l});
-    w.im = df_norm(DAcc{w.im.h, w.im.l});
-  }
-  // SX x + k y for a real k: one exact product, one TwoSum and the error terms
-  template <int SX>
-  static __device__ __forceinline__ DF uma1(const DF& x, const DF& k, const DF& y) {
-    const DAcc q = df_prod(y, k);
-    const float xh = SX > 0 ? x.h : -x.h, xl = SX > 0 ? x.l : -x.l;
-    const float s = fadd(q.s, xh);
-    const float bp = fsub(s, q.s);
-    const float err = fadd(fsub(q.s, fsub(s, bp)), fsub(xh, bp));
-    return DF{s, fadd(q.e, fadd(err, xl))};
-  }
-  template <int SX>
-  static __device__ __forceinline__ W uma(const W& x, const DF& k, const W& y) {
-    return W{uma1<SX>(x.re, k, y.re), uma1<SX>(x.im, k, y.im)};
-  }
-  static __device__ __forceinline__ W rscale(const DF& g, const W& x) {
-    return W{raw(df_prod(x.re, g)), raw(df_prod(x.im, g))};
-  }
-  // x + SY y: one TwoSum of the leading parts, the low parts and the error added
-  template <int SY>
-  static __device__ __forceinline__ DF uadd1(const DF& x, const DF& y) {
-    const float yh = SY > 0 ? y.h : -y.h, yl = SY > 0 ? y.l : -y.l;
-    const float s = fadd(x.h, yh);
-    const float bp = fsub(s, x.h);
-    const float err = fadd(fsub(x.h, fsub(s, bp)), fsub(yh, bp));
-    return DF{s, fadd(fadd(x.l, yl), err)};
-  }
-  template <int SY>
-  static __device__ __forceinline__ W uadd(const W& x, const W& y) {
-    return W{uadd1<SY>(x.re, y.re), uadd1<SY>(x.im, y.im)};
+  static __device__ __forceinline__ C kmul(const C& a, const C& b) { return ArDF::kmul(a, b); }
+  static __device__ __forceinline__ C cconst1() { return ArDF::cconst1(); }
+  static __device__ __forceinline__ W neg(const W& a) { return p2_neg(a); }
+  static __device__ __forceinline__ W mul_i(const W& a) {
+    return W{f2_swap(f2_conj(a.h)), f2_swap(f2_conj(a.l))};
   }
 };
-
+template <> struct Lz<ArDFP> {
+  using W = P2;
+  // c (re, im) = (re, im) * (cr, cr) + (im, re) * (-ci, ci)
+  struct K2 { P2 c, s; };
+  static __device__ __forceinline__ K2 k2(const DFK& c) {
+    return K2{P2{f2_dup(c.re.h), f2_dup(c.re.l)}, P2{f2_pack(-c.im.h, c.im.h), f2_pack(-c.im.l, c.im.l)}};
+  }
+  static __device__ __forceinline__ PAcc cprod(const K2& c, const W& a) {
+    PAcc A = p2_prod(a, c.c);
+    p2_mac(A, p2_swap(a), c.s);
+    return A;
+  }
+  static __device__ __forceinline__ void cmac(PAcc& A, const K2& c, const W& a) {
+    p2_mac(A, a, c.c);
+    p2_mac(A, p2_swap(a), c.s);
+  }
+  static __device__ __forceinline__ W cmul(const DFK& c, const W& a) { return p2_raw(cprod(k2(c), a)); }
+  static __device__ __forceinline__ W cmac2(const DFK& c0, const W& a, const DFK& c1, const W& b) {
+    PAcc A = cprod(k2(c0), a);
+    cmac(A, k2(c1), b);
+    return p2_raw(A);
+  }
+  static __device__ __forceinline__ W cmac4(const DFK* c, const W* a) {
+    PAcc A = cprod(k2(c[0]), a[0]);
+#pragma unroll
+    for (int i = 1; i < 4; ++i) cmac(A, k2(c[i]), a[i]);
+    return p2_raw(A);
+  }
+  static __device__ __forceinline__ DFK kmul(const DFK& a, const DFK& b) {
+    DFK r;
+    p2_lanes(cmul(a, P2{f2_pack(b.re.h, b.im.h), f2_pack(b.re.l, b.im.l)}), r.re, r.im);
+    return r;
+  }
+  static __device__ __forceinline__ W rmac2(const R2& c0, const W& a, const R2& c1, const W& b) {
+    PAcc A = p2_prod(a, P2{c0.h, c0.l});
+    p2_mac(A, b, P2{c1.h, c1.l});
+    return p2_raw(A);
+  }
+  static __device__ __forceinline__ void renorm(W& w) { w = p2_norm(PAcc{w.h, w.l}); }
+  // SX x + k y for a real k: one exact product, one TwoSum and the error
+  // terms, 12 packed operations (13 for SX < 0).  q is minus the product p.
+  template <int SX>
+  static __device__ __forceinline__ W uma(const W& x, const R2& k, const W& y) {
+    const f2 q = f2_mul(y.h, k.nh);
+    f2 e = f2_fma(y.h, k.h, q);
+    e = f2_fma(y.h, k.l, e);
+    e = f2_fma(y.l, k.h, e);
+    if (SX > 0) {
+      const f2 s = f2_sub(x.h, q);                        // p + x
+      const f2 bp = f2_add(s, q);                         // s - p
+      const f2 w = f2_add(f2_sub(s, bp), q);              // -(p - (s - bp))
+      const f2 err = f2_sub(f2_sub(x.h, bp), w);
+      return W{s, f2_add(e, f2_add(err, x.l))};
+    }
+    const f2 p = f2_mul(y.h, k.h);
+    const f2 s = f2_sub(p, x.h);
+    const f2 bp = f2_add(s, q);
+    const f2 err = f2_sub(f2_sub(p, f2_sub(s, bp)), f2_add(x.h, bp));
+    return W{s, f2_add(e, f2_sub(err, x.l))};
+  }
+  static __device__ __forceinline__ W rscale(const R2& g, const W& x) { return p2_raw(p2_prod(x, P2{g.h, g.l})); }
+  // x + SY y: one TwoSum of the leading parts, the low parts and the error added
+  template <int SY>
+  static __device__ __forceinline__ W uadd(const W& x, const W& y) {
+    if (SY > 0) {
+      const f2 s = f2_add(x.h, y.h);
+      const f2 bp = f2_sub(s, x.h);
+      const f2 err = f2_add(f2_sub(x.h, f2_sub(s, bp)), f2_sub(y.h, bp));
+      return W{s, f2_add(f2_add(x.l, y.l), err)};
+    }
+    const f2 s = f2_sub(x.h, y.h);
+    const f2 bp = f2_sub(s, x.h);
+    const f2 err = f2_sub(f2_sub(x.h, f2_sub(s, bp)), f2_add(y.h, bp));
+    return W{s, f2_add(f2_sub(x.l, y.l), err)};
+  }
+};
 template <class A>
 __device__ __forceinline__ void renorm(typename A::W& a) { Lz<A>::renorm(a); }
 
 template <class A> struct Re;
 template <> struct Re<ArF32> { static __device__ __forceinline__ float get(const float2& c) { return c.x; } };
 template <> struct Re<ArF64> { static __device__ __forceinline__ double get(const double2& c) { return c.x; } };
-template <> struct Re<ArDF> { static __device__ __forceinline__ DF get(const DFK& c) { return c.re; } };
+template <> struct Re<ArDFP> {
+  static __device__ __forceinline__ R2 get(const DFK& c) {
+    return R2{f2_dup(c.re.h), f2_dup(-c.re.h), f2_dup(c.re.l)};
+  }
+};
 
 // (a, b) <- (u00 a + u01 b, u10 a + u11 b)
 template <class A>
@@ -279,28 +352,35 @@ __device__ __forceinline__ void seg_expect(const TileGeom& G, uint64_t* bar, uin
 // compiled adjoint: gradient partials Im <lambda|G|psi>
 // ---------------------------------------------------------------------------
 template <class A> struct Dfc;
-template <> struct Dfc<ArF32> {
-  static __device__ __forceinline__ DFC get(const float2& w) { return DFC{DF{w.x, 0.f}, DF{w.y, 0.f}}; }
-};
 template <> struct Dfc<ArF64> {
   static __device__ __forceinline__ DFC get(const double2& w) { return DFC{d2df(w.x), d2df(w.y)}; }
-};
-template <> struct Dfc<ArDF> {
-  static __device__ __forceinline__ DFC get(const DFC& w) { return w; }
 };
 
 // Per-tile partial sums: double-float for complex128 (the products must keep
 // about 2^-46 relative accuracy), float32 for complex64 states.  Either is
-// added in float64 across tiles.
+// added in float64 across tiles.  T accumulates products of amplitudes (in
+// packed kernels one sum per component, added at the warp sum), B signed sums
+// of terms V.
 template <class A> struct GAcc {
   using T = DAcc;  // running sum (leading part, accumulated errors)
+  using B = DAcc;
   using V = DF;    // one term
   static __device__ __forceinline__ T zero() { return DAcc{0.f, 0.f}; }
+  static __device__ __forceinline__ B bzero() { return DAcc{0.f, 0.f}; }
+};
+template <> struct GAcc<ArDFP> {
+  using T = PAcc;
+  using B = DAcc;
+  using V = DF;
+  static __device__ __forceinline__ T zero() { return PAcc{0ull, 0ull}; }
+  static __device__ __forceinline__ B bzero() { return DAcc{0.f, 0.f}; }
 };
 template <> struct GAcc<ArF32> {
   using T = float;
+  using B = float;
   using V = float;
   static __device__ __forceinline__ T zero() { return 0.f; }
+  static __device__ __forceinline__ B bzero() { return 0.f; }
 };
 
 // acc += sign * Im(conj(l) p) = sign * (l.re p.im - l.im p.re)
@@ -313,6 +393,13 @@ __device__ __forceinline__ void gim_t(float& acc, const float2& l, const float2&
   acc = __fmaf_rn(s * l.x, p.y, acc);
   acc = __fmaf_rn(-s * l.y, p.x, acc);
 }
+__device__ __forceinline__ void gim_t(DAcc& acc, const double2& l, const double2& p, bool neg) {
+  gim_t(acc, Dfc<ArF64>::get(l), Dfc<ArF64>::get(p), neg);
+}
+__device__ __forceinline__ P2 p2_xor(const P2& a, f2 m) { return P2{a.h ^ m, a.l ^ m}; }
+__device__ __forceinline__ void gim_t(PAcc& acc, const P2& l, const P2& p, bool neg) {
+  p2_mac(acc, l, p2_xor(p2_swap(p), neg ? 0x0000000080000000ull : 0x8000000000000000ull));
+}
 // acc += sign * Re(conj(l) p) = sign * (l.re p.re + l.im p.im)
 __device__ __forceinline__ void gre_t(DAcc& acc, const DFC& l, const DFC& p, bool neg) {
   df_mac(acc, neg ? df_neg(l.re) : l.re, p.re);
@@ -323,25 +410,44 @@ __device__ __forceinline__ void gre_t(float& acc, const float2& l, const float2&
   acc = __fmaf_rn(s * l.x, p.x, acc);
   acc = __fmaf_rn(s * l.y, p.y, acc);
 }
+__device__ __forceinline__ void gre_t(DAcc& acc, const double2& l, const double2& p, bool neg) {
+  gre_t(acc, Dfc<ArF64>::get(l), Dfc<ArF64>::get(p), neg);
+}
+__device__ __forceinline__ void gre_t(PAcc& acc, const P2& l, const P2& p, bool neg) {
+  p2_mac(acc, l, p2_xor(p, neg ? 0x8000000080000000ull : 0ull));
+}
 template <class A>
 __device__ __forceinline__ void gim(typename GAcc<A>::T& acc, const typename A::W& l, const typename A::W& p, bool neg) {
-  if constexpr (sizeof(typename GAcc<A>::T) == sizeof(float)) gim_t(acc, l, p, neg);
-  else gim_t(acc, Dfc<A>::get(l), Dfc<A>::get(p), neg);
+  gim_t(acc, l, p, neg);
 }
 template <class A>
 __device__ __forceinline__ void gre(typename GAcc<A>::T& acc, const typename A::W& l, const typename A::W& p, bool neg) {
-  if constexpr (sizeof(typename GAcc<A>::T) == sizeof(float)) gre_t(acc, l, p, neg);
-  else gre_t(acc, Dfc<A>::get(l), Dfc<A>::get(p), neg);
+  gre_t(acc, l, p, neg);
+}
+// the scalar value of an accumulator
+__device__ __forceinline__ float gval(float a) { return a; }
+__device__ __forceinline__ DAcc gval(const DAcc& a) { return a; }
+__device__ __forceinline__ DAcc gval(const PAcc& a) {
+  DF x, y;
+  p2_lanes(P2{a.s, a.e}, x, y);
+  DAcc A{x.h, x.l};
+  df_acc(A, y);
+  return A;
 }
 
 // One term w = Im(conj(l) p), shared by every Z / P1 partial of a merged
 // diagonal run (those partials are signed sums of the same w_j).
+__device__ __forceinline__ float gterm(float a) { return a; }
+__device__ __forceinline__ DF gterm(const DAcc& a) { return df_norm(a); }
 template <class A>
 __device__ __forceinline__ typename GAcc<A>::V wim(const typename A::W& l, const typename A::W& p) {
   typename GAcc<A>::T a = GAcc<A>::zero();
   gim<A>(a, l, p, false);
-  if constexpr (sizeof(typename GAcc<A>::T) == sizeof(float)) return a;
-  else return df_norm(a);
+  return gterm(gval(a));
+}
+template <>
+__device__ __forceinline__ DF wim<ArDFP>(const P2& l, const P2& p) {
+  return df_norm(gval(p2_prod(l, p2_xor(p2_swap(p), 0x8000000000000000ull))));
 }
 __device__ __forceinline__ void wadd(DAcc& acc, const DF& w, bool neg) { df_acc(acc, neg ? df_neg(w) : w); }
 __device__ __forceinline__ void wadd(float& acc, float w, bool neg) { acc = neg ? acc - w : acc + w; }
@@ -401,6 +507,10 @@ __device__ __forceinline__ void gflush4(const DAcc& a0, const DAcc& a1, const DA
   k = df_add(k, shfl_df(k, 1));
   double* s = u16 ? (u8 ? s3 : s2) : (u8 ? s1 : s0);
   if ((lane & 7u) == 0 && s) slot_add(s, k);
+}
+__device__ __forceinline__ void gflush4(const PAcc& a0, const PAcc& a1, const PAcc& a2, const PAcc& a3, double* s0,
+                                        double* s1, double* s2, double* s3) {
+  gflush4(gval(a0), gval(a1), gval(a2), gval(a3), s0, s1, s2, s3);
 }
 __device__ __forceinline__ void gflush4(float a0, float a1, float a2, float a3, double* s0, double* s1, double* s2,
                                         double* s3) {
@@ -476,27 +586,27 @@ __device__ __forceinline__ DF pnorm2(const DFC& v) {
   df_mac(a, v.im, v.im);
   return df_norm(a);
 }
+__device__ __forceinline__ DF pnorm2(const double2& v) { return pnorm2(Dfc<ArF64>::get(v)); }
+__device__ __forceinline__ DF pnorm2(const P2& v) { return df_norm(gval(p2_prod(v, v))); }
 __device__ __forceinline__ float pnorm2(const float2& v) { return __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y)); }
 template <class A>
-__device__ __forceinline__ typename GAcc<A>::V pn2(const typename A::W& w) {
-  if constexpr (sizeof(typename GAcc<A>::T) == sizeof(float)) return pnorm2(w);
-  else return pnorm2(Dfc<A>::get(w));
-}
+__device__ __forceinline__ typename GAcc<A>::V pn2(const typename A::W& w) { return pnorm2(w); }
 
 // lambda_j accumulated per component: double-float for complex128 states,
 // float32 for complex64.
-template <class A> struct LAcc {
+template <class A> struct LAcc;
+template <> struct LAcc<ArF64> {
   DAcc re, im;
-  __device__ __forceinline__ void init(const typename A::W& w) {
-    const DFC v = Dfc<A>::get(w);
+  __device__ __forceinline__ void init(const double2& w) {
+    const DFC v = Dfc<ArF64>::get(w);
     re = DAcc{v.re.h, v.re.l};
     im = DAcc{v.im.h, v.im.l};
   }
   __device__ __forceinline__ void zero() { re = im = DAcc{0.f, 0.f}; }
   // += c * sign * i^PH * w
   template <int PH>
-  __device__ __forceinline__ void add(const typename A::W& w, const DF& c, bool neg) {
-    const DFC v = Dfc<A>::get(w);
+  __device__ __forceinline__ void add(const double2& w, const DF& c, bool neg) {
+    const DFC v = Dfc<ArF64>::get(w);
     DF vr = v.re, vi = v.im;
     if (PH & 1) { const DF t = vr; vr = df_neg(vi); vi = t; }
     if (PH & 2) { vr = df_neg(vr); vi = df_neg(vi); }
@@ -504,12 +614,22 @@ template <class A> struct LAcc {
     df_mac(re, vr, c);
     df_mac(im, vi, c);
   }
-  __device__ __forceinline__ typename A::W out() const;
+  __device__ __forceinline__ double2 out() const {
+    return make_double2(df2d(df_norm(re)), df2d(df_norm(im)));
+  }
 };
-template <> __device__ __forceinline__ DFC LAcc<ArDF>::out() const { return DFC{df_norm(re), df_norm(im)}; }
-template <> __device__ __forceinline__ double2 LAcc<ArF64>::out() const {
-  return make_double2(df2d(df_norm(re)), df2d(df_norm(im)));
-}
+template <> struct LAcc<ArDFP> {
+  PAcc a;
+  __device__ __forceinline__ void init(const P2& w) { a = PAcc{w.h, w.l}; }
+  __device__ __forceinline__ void zero() { a = PAcc{0ull, 0ull}; }
+  template <int PH>
+  __device__ __forceinline__ void add(const P2& w, const DF& c, bool neg) {
+    const bool n = neg != ((PH & 2) != 0);  // the sign goes to the coefficient
+    const float ch = n ? -c.h : c.h, cl = n ? -c.l : c.l;
+    p2_mac(a, (PH & 1) ? ArDFP::mul_i(w) : w, P2{f2_dup(ch), f2_dup(cl)});
+  }
+  __device__ __forceinline__ P2 out() const { return p2_norm(a); }
+};
 template <> struct LAcc<ArF32> {
   float re, im;
   __device__ __forceinline__ void init(const float2& w) { re = w.x; im = w.y; }

@@ -135,7 +135,7 @@ std::string pauli_source(const char* aname, int k, int b, const std::vector<JWor
       auto it = walsh.find(zr);
       if (it == walsh.end()) {
         const std::string sn = "d" + std::to_string(uid++);
-        o << "    lqs::jit::GAcc<A>::T " << sn << " = lqs::jit::GAcc<A>::zero();\n";
+        o << "    lqs::jit::GAcc<A>::B " << sn << " = lqs::jit::GAcc<A>::bzero();\n";
         for (int e = 0; e < R; ++e)
           o << "    lqs::jit::wadd(" << sn << ", p" << e << ", " << ((__builtin_popcount(e & zr) & 1) ? "true" : "false")
             << ");\n";
@@ -271,7 +271,7 @@ std::string pauli_source(const char* aname, int k, int b, const std::vector<JWor
     for (auto& W : ws)
       if (!W.xl) any_diag = true;
     if (any_diag) {
-      for (int e = 0; e < R; ++e) o << "    lqs::jit::GAcc<A>::T c" << e << " = lqs::jit::GAcc<A>::zero();\n";
+      for (int e = 0; e < R; ++e) o << "    lqs::jit::GAcc<A>::B c" << e << " = lqs::jit::GAcc<A>::bzero();\n";
       for (int w = 0; w < nw; ++w) {
         const JWord& W = ws[w];
         if (W.xl) continue;
@@ -323,7 +323,7 @@ std::string pauli_source(const char* aname, int k, int b, const std::vector<JWor
     << "typedef unsigned char uint8_t;\ntypedef signed char int8_t;\ntypedef short int16_t;\ntypedef unsigned short uint16_t;\n"
        "typedef unsigned int uint32_t;\ntypedef unsigned long long uint64_t;\n"
     << "#include \"tile.cuh\"\n#include \"jit_dev.cuh\"\n"
-    << "typedef " << aname << " A;\n"
+    << "typedef " << jit_policy(aname) << " A;\n"
     << "struct PArgs {\n  lqs::TileGeom g;\n  lqs::jit::PCoef<A>::T c[" << std::max(nw, 1) << "];\n};\n"
     << "extern \"C\" __global__ void __launch_bounds__(256, 2)\n"
     << kname << "(const A::S* __restrict__ psi, A::S* __restrict__ lam, const __grid_constant__ PArgs P, "
