@@ -11,6 +11,7 @@
 // between the streams.
 #include <algorithm>
 #include <string>
+#include <type_traits>
 
 #include "arith.cuh"
 #include "lqs_internal.cuh"
@@ -214,6 +215,65 @@ __global__ void __launch_bounds__(kThreads) k_dense2(typename A::S* __restrict__
   }
 }
 
+// Double-float 4x4 update, both components of an amplitude per instruction.
+// A complex coefficient c acts as (re, im) * (cr, cr) + (im, re) * (-ci, ci):
+// the host lays out those pairs and the negated leading parts (q = -p makes a
+// product's error term one fma), so they cost no instruction here.  12 FP32
+// operations per real product as in the scalar form, half the instructions:
+// the float32 pipe is the bound (28 qubits, per gate: 2.07 -> 1.88 ms; one
+// read and write of the state take 1.27 ms).
+struct K4 { unsigned long long ch, cn, cl, sh, sn, sl; };  // (cr, cr): leading, negated, low; (-ci, ci) likewise
+struct Mat4P { K4 c[16]; };
+
+// A + a * (h, l) with n = -h; see df_mac
+__device__ __forceinline__ void k4_mac(PAcc& A, const P2& a, f2 h, f2 n, f2 l) {
+  const f2 q = f2_mul(a.h, n);  // minus the product
+  f2 e = f2_fma(a.h, h, q);
+  e = f2_fma(a.h, l, e);
+  e = f2_fma(a.l, h, e);
+  const f2 s = f2_sub(A.s, q);
+  const f2 bp = f2_sub(s, A.s);
+  const f2 err = f2_sub(f2_sub(A.s, f2_sub(s, bp)), f2_add(q, bp));
+  A.s = s;
+  A.e = f2_add(A.e, f2_add(err, e));
+}
+
+__global__ void __launch_bounds__(kThreads) k_dense2_df(double2* __restrict__ psi, Geom G,
+                                                        const __grid_constant__ Mat4P M) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g < G.ngroups; g += stride) {
+    const uint64_t base = group_base(G, g);
+    const uint64_t id[4] = {base, base | G.b1, base | G.b0, base | G.b0 | G.b1};
+    double2 s[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) s[r] = psi[id[r]];
+    P2 x[4], y[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const DF re = d2df(s[r].x), im = d2df(s[r].y);
+      x[r] = P2{f2_pack(re.h, im.h), f2_pack(re.l, im.l)};
+      y[r] = p2_swap(x[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const K4* c = &M.c[4 * r];
+      f2 q = f2_mul(x[0].h, c[0].cn);
+      f2 e = f2_fma(x[0].h, c[0].ch, q);
+      e = f2_fma(x[0].h, c[0].cl, e);
+      PAcc A{f2_neg(q), f2_fma(x[0].l, c[0].ch, e)};
+      k4_mac(A, y[0], c[0].sh, c[0].sn, c[0].sl);
+#pragma unroll
+      for (int k = 1; k < 4; ++k) {
+        k4_mac(A, x[k], c[k].ch, c[k].cn, c[k].cl);
+        k4_mac(A, y[k], c[k].sh, c[k].sn, c[k].sl);
+      }
+      DF re, im;
+      p2_lanes(p2_raw(A), re, im);
+      psi[id[r]] = make_double2(df2d(re), df2d(im));
+    }
+  }
+}
+
 template <class A>
 __global__ void __launch_bounds__(kThreads) k_diag2(typename A::S* __restrict__ psi, Geom G, typename A::C d0,
                                                     typename A::C d1, typename A::C d2, typename A::C d3) {
@@ -254,6 +314,12 @@ static unsigned grid_for(const SV* sv, uint64_t work) {
 
 template <class A>
 static typename A::C cc(const KOp& op, int i) { return A::cconst(op.m[2 * i], op.m[2 * i + 1]); }
+
+static K4 k4_const(double re, double im) {
+  const DF r = split_const(re), i = split_const(im);
+  auto two = [](float lo, float hi) { return (unsigned long long)f_bits(lo) | (unsigned long long)f_bits(hi) << 32; };
+  return K4{two(r.h, r.h), two(-r.h, -r.h), two(r.l, r.l), two(-i.h, i.h), two(i.h, -i.h), two(-i.l, i.l)};
+}
 
 static const char* gate_kernel_name(int kind) {
   static const char* names[] = {"k_phase", "k_diag1", "k_anti1", "k_swap", "k_dense1", "k_dense1r", "k_dense2",
@@ -305,11 +371,17 @@ static int launch_gate_t(SV* sv, const KOp& op, int arith) {
     }
     case K_DENSE2: {
       Geom G = make_geom(n, op, true);
-      Mat4<typename A::C> M;
-      for (int i = 0; i < 16; ++i) M.c[i] = cc<A>(op, i);
       unsigned grid = (unsigned)std::max<uint64_t>(
           1, std::min<uint64_t>((G.ngroups + kThreads - 1) / kThreads, (uint64_t)std::max(sv->sms, 1) * 8));
-      k_dense2<A><<<grid, kThreads, 0, st>>>(psi, G, M);
+      if constexpr (std::is_same<A, ArDF>::value) {
+        Mat4P M;
+        for (int i = 0; i < 16; ++i) M.c[i] = k4_const(op.m[2 * i], op.m[2 * i + 1]);
+        k_dense2_df<<<grid, kThreads, 0, st>>>(psi, G, M);
+      } else {
+        Mat4<typename A::C> M;
+        for (int i = 0; i < 16; ++i) M.c[i] = cc<A>(op, i);
+        k_dense2<A><<<grid, kThreads, 0, st>>>(psi, G, M);
+      }
       break;
     }
     case K_DIAG2: {

@@ -60,52 +60,15 @@ template <class A> struct Lz {
     return r;
   }
 };
-// Double-float amplitudes of compiled segments, two floats to a register pair
-// (arith.cuh f2): the leading parts of (re, im) and their low parts.  Every
-// operation runs on both components at once, in the order and with the
-// roundings of the scalar forms (arith.cuh df_prod, df_mac), so results are
-// those of ArDF bit for bit.
-struct P2 { f2 h, l; };   // two double-floats
-struct PAcc { f2 s, e; };  // two accumulators (leading sums, collected errors)
-__device__ __forceinline__ P2 p2_raw(const PAcc& a) { return P2{a.s, a.e}; }
-__device__ __forceinline__ P2 p2_neg(const P2& a) { return P2{f2_neg(a.h), f2_neg(a.l)}; }
-__device__ __forceinline__ P2 p2_swap(const P2& a) { return P2{f2_swap(a.h), f2_swap(a.l)}; }
-__device__ __forceinline__ P2 p2_norm(const PAcc& a) {
-  const f2 h = f2_add(a.s, a.e);
-  return P2{h, f2_sub(a.e, f2_sub(h, a.s))};
-}
-__device__ __forceinline__ PAcc p2_prod(const P2& a, const P2& c) {
-  const f2 p = f2_mul(a.h, c.h);
-  f2 e = f2_fma(a.h, c.h, f2_neg(p));
-  e = f2_fma(a.h, c.l, e);
-  e = f2_fma(a.l, c.h, e);
-  return PAcc{p, e};
-}
-__device__ __forceinline__ void p2_acc(PAcc& A, f2 x, f2 xe) {  // A += x + xe, TwoSum on the leading parts
-  const f2 s = f2_add(A.s, x);
-  const f2 bp = f2_sub(s, A.s);
-  const f2 err = f2_add(f2_sub(A.s, f2_sub(s, bp)), f2_sub(x, bp));
-  A.s = s;
-  A.e = f2_add(A.e, f2_add(err, xe));
-}
-__device__ __forceinline__ void p2_mac(PAcc& A, const P2& a, const P2& c) {
-  const PAcc q = p2_prod(a, c);
-  p2_acc(A, q.s, q.e);
-}
-// lane 0 / lane 1 as scalar double-floats
-__device__ __forceinline__ void p2_lanes(const P2& a, DF& x, DF& y) {
-  f2_unpack(a.h, x.h, y.h);
-  f2_unpack(a.l, x.l, y.l);
-}
 }  // namespace jit
 
 // 128-bit shared-memory and global accesses of working amplitudes.
-__device__ __forceinline__ void st_w(jit::P2* p, const jit::P2& v) {
+__device__ __forceinline__ void st_w(P2* p, const P2& v) {
   *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v.h, v.l);
 }
-__device__ __forceinline__ jit::P2 ld_w(const jit::P2* p) {
+__device__ __forceinline__ P2 ld_w(const P2* p) {
   const ulonglong2 f = *reinterpret_cast<const ulonglong2*>(p);
-  return jit::P2{f.x, f.y};
+  return P2{f.x, f.y};
 }
 
 namespace jit {
