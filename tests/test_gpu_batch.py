@@ -113,3 +113,23 @@ def test_batch_autotune_keeps_a_shape_per_qubit_count():
         assert abs(ei - oracle.energy(c, t)) <= 2 * c64_rel_bound(len(c.ops)) * scale
         np.testing.assert_allclose(gi, oracle.param_shift_grad(c, t), rtol=0,
                                    atol=4 * c64_rel_bound(2 * len(c.ops)) * scale)
+
+
+@pytest.mark.parametrize("dtype,arith", [("c128", "df"), ("c128", "f64"), ("c64", "f32")])
+@pytest.mark.parametrize("n", [5, 7, 8, 9, 11, 12, 13, 15])
+def test_batch_whole_gate_set(dtype, arith, n):
+    """Every gate class and generator in the batch kernel, on tiles too small for register programs (5), with idle
+    threads (7-11), of one tile (12) and of several, with Pauli words on register, thread and outside bits; same
+    tolerances as above."""
+    import paper_2508_13615_gb300 as L
+    set_mode(arith)
+    circs = [W.random_circuit(n, 45, seed=300 + n), W.random_circuit(n, 30, seed=400 + n)]
+    words = W.tfim(n) + [W.pauli_word(0.7, {0: "Y", n - 1: "Y"}), W.pauli_word(-0.4, {1: "X", n - 2: "Z"}),
+                         W.pauli_word(0.2, {0: "X", 1: "Y", n - 1: "Z"}), W.pauli_word(1.5, {})]
+    e, g = L.lqs_batch_run(circs, [words, words], dtype)
+    scale = sum(abs(w.coeff) for w in words)
+    for c, ei, gi in zip(circs, e, g):
+        tol_e, tol_g = (1e-10, 1e-10) if dtype == "c128" else (2 * c64_rel_bound(len(c.ops)) * scale,
+                                                                4 * c64_rel_bound(2 * len(c.ops)) * scale)
+        assert abs(ei - oracle.energy(c, words)) <= tol_e
+        np.testing.assert_allclose(gi, oracle.param_shift_grad(c, words), rtol=0, atol=tol_g)
