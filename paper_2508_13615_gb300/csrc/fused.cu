@@ -8,8 +8,11 @@
 // play the role of the local qubits, and choosing them per segment lets the
 // "non-local" gates become local too.
 #include <algorithm>
+#include <iterator>
+#include <mutex>
 #include <string>
 #include <type_traits>
+#include <unordered_map>
 
 #include "arith.cuh"
 #include "jit.h"
@@ -20,9 +23,10 @@
 // Dense work per segment: a compiled segment is straight-line code, and one
 // whose dense updates add up past this weight (4 per two-qubit dense op, 1
 // per one-qubit dense op; diagonal and permutation ops are free) spends more
-// in instruction fetch than a further pass costs.
+// in instruction fetch than a further pass costs.  30-qubit 10-layer ansatz,
+// complex128: caps of 8 / 12 / 16 / 24 / 40 ran 451 / 418 / 426 / 453 / 510 ms.
 #ifndef LQS_SEGMENT_DENSE_CAP
-#define LQS_SEGMENT_DENSE_CAP 16
+#define LQS_SEGMENT_DENSE_CAP 12
 #endif
 // complex64 segments carry float32 arithmetic, several times less code per op
 #ifndef LQS_SEGMENT_DENSE_CAP_C64
@@ -58,6 +62,10 @@ int resolve_cfg(int n, int dtype, const lqs_fuse_cfg* cfg, PlanCfg& pc, int* ari
   if (pc.b < std::max(bmin, 1) || pc.b > pc.k - 2)
     return set_error(LQS_ERR_ARG, "low_qubits must be in [1, tile_qubits - 2]");
   if (pc.max_ops < 1) return set_error(LQS_ERR_ARG, "max_ops must be positive");
+  // complex128 only: another order of commuting gates rounds differently, far
+  // below double precision but by up to the last float32 bit in complex64,
+  // whose energies and gradients are to stay what program order gives
+  pc.search = dtype == LQS_C128 && pc.dense_cap > 0 && pc.k == reg_tile_qubits(dtype);
   if (n <= pc.k) {  // the whole state is one tile
     pc.k = n;
     pc.b = n;
@@ -84,59 +92,152 @@ static int coef_count(const KOp& o) {
 // planner
 // ---------------------------------------------------------------------------
 //
-// Greedy in program order.  A segment starts with the low b qubits in its
-// tile.  Each not-yet-scheduled op is taken if (1) no earlier unscheduled op
-// shares a wire with it ("blocked" wires), so moving it ahead of those ops
-// only passes gates on disjoint wires, which commute, and (2) its
-// non-diagonal targets fit the tile, adding qubits while fewer than k are
-// used.  Diagonal ops and controls need no tile qubit.  An op that is not
-// taken blocks its wires for the rest of the segment.
+// A segment executes remaining ops that (1) commute with all earlier ops it
+// leaves behind and (2) have their non-diagonal targets in the segment's tile.
+// Diagonal ops and controls need no tile qubit.  Ops on disjoint wires
+// commute; searched plans also let ops pass each other when every wire they
+// share is one that both leave in the Z basis (controls, diagonal targets).
 static int dense_weight(const KOp& o) {
   return o.kind == K_DENSE2 ? 4 : (o.kind == K_DENSE1 || o.kind == K_DENSE1R) ? 1 : 0;
 }
 
-int plan_segments(int n, const std::vector<KOp>& ops, const PlanCfg& pc, std::vector<Segment>& segs) {
+
+namespace {
+struct POp {
+  uint64_t x, z;  // wires it must keep its order on / may pass other z wires on
+  uint64_t t;     // qubits it needs in the tile
+  int nc, dense;
+};
+
+// The remaining ops (indices `rem`, in order) that one segment with tile Q
+// executes; with `grow`, Q gains qubits in program order while it holds fewer
+// than k.  Returns the weight of the executed ops.
+int fill_segment(const std::vector<POp>& ops, const std::vector<int>& rem, const PlanCfg& pc, int k, uint64_t all,
+                 bool grow, uint64_t& Q, std::vector<int>* out) {
+  uint64_t bx = 0, bz = 0;  // wires of the ops left behind
+  int n_ops = 0, ncoef = 0, dense = 0, weight = 0;
+  for (int i : rem) {
+    const POp& o = ops[(size_t)i];
+    if (!(o.x & (bx | bz)) && !(o.z & bx)) {
+      const uint64_t need = o.t & ~Q;
+      if ((!need || (grow && __builtin_popcountll(Q | need) <= k)) && n_ops < pc.max_ops &&
+          ncoef + o.nc <= kMaxTileCoef && (pc.dense_cap <= 0 || dense + o.dense <= pc.dense_cap || !n_ops)) {
+        Q |= need;
+        ++n_ops;
+        ncoef += o.nc;
+        dense += o.dense;
+        weight += o.t ? 8 : 1;
+        if (out) out->push_back(i);
+        continue;
+      }
+    }
+    bx |= o.x;
+    bz |= o.z;
+    if (bx == all) break;
+  }
+  return weight;
+}
+
+// One plan.  Without search each segment takes qubits in program order.  With
+// it every window of neighbouring qubits is tried too, and the tile that
+// executes the most is improved by exchanging one qubit at a time.  Layers
+// with a CNOT ladder advance in skewed windows this way (half the qubits per
+// layer, two to five layers per pass): 30-qubit 10-layer ansatz, complex128 33
+// -> 27 passes (21 with a dense cap of 16) and 444 -> 418 ms; 24-qubit
+// universal circuit 55 -> 23 and 6.29 -> 5.29 ms.
+int make_plan(int n, const std::vector<POp>& ops, const PlanCfg& pc, bool search, std::vector<Segment>& segs) {
   const int k = std::min(pc.k, n), b = std::min(pc.b, k);
   const uint64_t all = n >= 64 ? ~0ull : ((1ull << n) - 1);
   const uint64_t low = b >= 64 ? ~0ull : ((1ull << b) - 1);
-  std::vector<char> done(ops.size(), 0);
-  size_t remaining = ops.size(), first = 0;
+  auto padded = [&](uint64_t Q) {
+    for (int q = b; q < n && __builtin_popcountll(Q) < k; ++q) Q |= 1ull << q;
+    return Q;
+  };
+  std::vector<int> rem(ops.size());
+  for (size_t i = 0; i < ops.size(); ++i) rem[i] = (int)i;
   segs.clear();
-  while (remaining) {
-    while (done[first]) ++first;
+  while (!rem.empty()) {
     Segment seg;
-    uint64_t Q = low, blocked = 0;
-    int ncoef = 0, dense = 0;
-    for (size_t i = first; i < ops.size() && blocked != all; ++i) {
-      if (done[i]) continue;
-      const KOp& o = ops[i];
-      const uint64_t wires = o.wire_mask();
-      if (wires & blocked) {
-        blocked |= wires;
-        continue;
+    uint64_t Q = low;
+    int best = fill_segment(ops, rem, pc, k, all, true, Q, search ? nullptr : &seg.ops);
+    Q = padded(Q);
+    if (search) {
+      auto weigh = [&](uint64_t T) { return fill_segment(ops, rem, pc, k, all, false, T, nullptr); };
+      best = std::max(best, weigh(Q));
+      for (int s = b; s + (k - b) <= n; ++s) {
+        const uint64_t T = low | (((1ull << (k - b)) - 1) << s);
+        const int w = weigh(T);
+        if (w > best) best = w, Q = T;
       }
-      const uint64_t need = o.tile_mask() & ~Q;
-      const int nc = coef_count(o);
-      const int dw = dense_weight(o);
-      const bool fits = __builtin_popcountll(Q | need) <= k && (int)seg.ops.size() < pc.max_ops &&
-                        ncoef + nc <= kMaxTileCoef &&
-                        (pc.dense_cap <= 0 || dense + dw <= pc.dense_cap || seg.ops.empty());
-      if (fits) {
-        Q |= need;
-        seg.ops.push_back((int)i);
-        done[i] = 1;
-        --remaining;
-        ncoef += nc;
-        dense += dw;
-      } else {
-        blocked |= wires;
+      for (int round = 0; round < 4; ++round) {
+        uint64_t top = Q;
+        for (int i = b; i < n; ++i) {
+          if (!((Q >> i) & 1)) continue;
+          for (int j = b; j < n; ++j) {
+            if ((Q >> j) & 1) continue;
+            const uint64_t T = (Q & ~(1ull << i)) | (1ull << j);
+            const int w = weigh(T);
+            if (w > best) best = w, top = T;
+          }
+        }
+        if (top == Q) break;
+        Q = top;
       }
     }
-    if (seg.ops.empty()) return set_error(LQS_ERR_ARG, "internal: planner made no progress");
-    for (int q = b; q < n && __builtin_popcountll(Q) < k; ++q) Q |= 1ull << q;  // pad to exactly k qubits
     seg.qmask = Q;
+    if (search) fill_segment(ops, rem, pc, k, all, false, Q, &seg.ops);
+    if (seg.ops.empty()) return set_error(LQS_ERR_ARG, "internal: planner made no progress");
+    std::vector<int> left;
+    left.reserve(rem.size() - seg.ops.size());
+    std::set_difference(rem.begin(), rem.end(), seg.ops.begin(), seg.ops.end(), std::back_inserter(left));
+    rem.swap(left);
     segs.push_back(std::move(seg));
   }
+  return LQS_OK;
+}
+
+// Plans with a search cost 2-20 ms of host time (300-900 ops), so they are
+// kept by structure: everything the plan depends on, never an address.
+constexpr size_t kMaxSearchedPlans = 256;
+std::mutex g_search_mu;
+std::unordered_map<std::string, std::vector<Segment>> g_searched;
+}  // namespace
+
+int plan_segments(int n, const std::vector<KOp>& ops, const PlanCfg& pc, std::vector<Segment>& segs) {
+  std::vector<POp> po(ops.size());
+  auto set_pass = [&](bool commute) {
+    for (size_t i = 0; i < ops.size(); ++i) {
+      const uint64_t t = ops[i].tile_mask(), w = ops[i].wire_mask();
+      po[i] = POp{commute ? t : w, commute ? w & ~t : 0, t, coef_count(ops[i]), dense_weight(ops[i])};
+    }
+  };
+  set_pass(false);
+  if (!pc.search) return make_plan(n, po, pc, false, segs);
+  std::string key;
+  const int hdr[5] = {n, pc.k, pc.b, pc.max_ops, pc.dense_cap};
+  key.append(reinterpret_cast<const char*>(hdr), sizeof hdr);
+  for (const POp& o : po) {
+    const uint64_t rec[3] = {o.x, o.t, (uint64_t)o.nc << 32 | (uint64_t)o.dense};
+    key.append(reinterpret_cast<const char*>(rec), sizeof rec);
+  }
+  {
+    std::lock_guard<std::mutex> lk(g_search_mu);
+    auto it = g_searched.find(key);
+    if (it != g_searched.end()) {
+      segs = it->second;
+      return LQS_OK;
+    }
+  }
+  LQS_TRY(make_plan(n, po, pc, false, segs));
+  if (segs.size() > 1) {
+    std::vector<Segment> alt;
+    set_pass(true);
+    LQS_TRY(make_plan(n, po, pc, true, alt));
+    if (alt.size() < segs.size()) segs.swap(alt);
+  }
+  std::lock_guard<std::mutex> lk(g_search_mu);
+  if (g_searched.size() >= kMaxSearchedPlans) g_searched.clear();
+  g_searched.emplace(std::move(key), segs);
   return LQS_OK;
 }
 

@@ -862,21 +862,22 @@ int note_reg_prog(int n, int dtype, int arith, const std::vector<KOp>& ops, cons
 // ---------------------------------------------------------------------------
 // compiled adjoint (reverse sweep over psi and lambda)
 // ---------------------------------------------------------------------------
-// The kernel holds two states in registers and four tiles in shared memory
-// (incoming psi and lambda, two exchange buffers), so its tiles are smaller
-// than the forward kernel's: 2^11 amplitudes for both dtypes.
-// Shape of the compiled adjoint: register bits per state and thread bits.
-// Measured on GB300 (24-qubit ansatz): complex128 runs fastest with 4
-// amplitudes of each state per thread and 512 threads, one CTA per SM (half
-// the code per op of 8 amplitudes; 256 threads were 3% slower), complex64
-// with 16 per state and 128 threads, three CTAs per SM.
-#ifndef LQS_ADJ_THREAD_BITS_C128
-#define LQS_ADJ_THREAD_BITS_C128 9
-#endif
+// The kernel holds a tile of 2^11 amplitudes of psi and of lambda in
+// registers: complex128 in 256 threads (8 of each state per thread), complex64
+// in 128 (16 per thread), one buffer per tile, two and four CTAs per SM.
 static void adj_shape(int dtype, int* r, int* tb) {
-  *r = dtype == LQS_C64 ? 4 : 2;
-  *tb = dtype == LQS_C64 ? 7 : LQS_ADJ_THREAD_BITS_C128;
+  *r = dtype == LQS_C64 ? 4 : 3;
+  *tb = dtype == LQS_C64 ? 7 : 8;
 }
+// Dense work per reverse segment (complex128): an op costs about four times
+// its forward code (two states and a partial), and the search for fuller
+// segments makes them longer than the instruction cache holds.  24-qubit
+// 8-layer gradient: 45 ms without a cap (25 ms with the program-order plan);
+// caps of 4 / 6 / 8 / 12 / 16 / 24 on kernels with two CTAs per SM 25.8 / 22.6 /
+// 21.9 / 22.0 / 21.6 / 22.1 ms.
+#ifndef LQS_ADJOINT_DENSE_CAP
+#define LQS_ADJOINT_DENSE_CAP 16
+#endif
 int adjoint_tile_qubits(int dtype) {
   int r, tb;
   adj_shape(dtype, &r, &tb);
@@ -930,6 +931,10 @@ static int adj_prepare_t(int n, int dtype, const std::vector<KOp>& rev, std::vec
   pc.k = k;
   pc.b = b;
   pc.max_ops = kMaxTileOps;
+  if (dtype == LQS_C128) {  // complex64 keeps program order (resolve_cfg)
+    pc.search = true;
+    pc.dense_cap = LQS_ADJOINT_DENSE_CAP;
+  }
   std::vector<Segment> segs;
   LQS_TRY(plan_segments(n, rev, pc, segs));
   for (const Segment& sg : segs) LQS_TRY(adj_build(n, rev, sg, k, b, r, progs));

@@ -119,8 +119,7 @@ class SegGen {
   // adjoint: the kernel carries psi and lambda (same layout and renamings),
   // and ops with a gradient slot (and K_GRAD partials) add Im<lambda|G|psi>.
   SegGen(int k, int b, int r, const char* aname, int amp_bytes, bool adjoint)
-      : k_(k), b_(b), r_(r), R_(1 << r), aname_(aname), sz_(amp_bytes), adj_(adjoint),
-        xpair_(adjoint && amp_bytes == 16) {}
+      : k_(k), b_(b), r_(r), R_(1 << r), aname_(aname), sz_(amp_bytes), adj_(adjoint) {}
   void set_folds(const TFold* f) { folds_ = f; }
 
   // Returns false (with a reason) for a program this generator does not take.
@@ -132,11 +131,6 @@ class SegGen {
   int sz_;
   bool adj_;
   const char* pfx_ = "v";       // variables of the state being emitted ("v" psi, "u" lambda)
-  int xb_ = 0;                  // exchange buffer of the next exchange (they alternate)
-  // complex128 adjoint: psi and lambda cross each exchange together, through
-  // the pair XA/XB or XC/XD (alternating), under one barrier
-  bool xpair_ = false;
-  int xp_ = 0;
   int next_bar_ = 1;            // next free named barrier id in this tile iteration (0 is the block barrier)
   int slot_[4] = {0, 0, 0, 0};  // register slot m -> local position
   int thr_[16] = {0};           // thread bit m -> local position
@@ -187,7 +181,7 @@ class SegGen {
   // gradient partials (seg_scales) and folds into a diagonal run or a final
   // scale; launches whose product of m00's is too small run elsewhere.
   bool unit_adj() const { return adj_ && aname_ == std::string("lqs::ArDF"); }
-  int npf_ = 0;  // forward: places where the next tile's load could start (after each exchange)
+  int npf_ = 0;  // places where the next tile's load could start (after each exchange)
   void flush_pending(bool all);
   // runs f once per state, with V() naming that state's variables
   template <class F>
@@ -506,13 +500,11 @@ bool SegGen::exchange_safe(int buf, const std::vector<uint8_t>& wown) const {
 }
 
 void SegGen::emit_layout(const TOp& t) {
-  // Each state is written in the current layout and read back in the new one.
-  // Forward programs use the tile's one buffer; the ordering check below adds a
-  // block barrier before the writes when the previous exchange's readers are
-  // not ordered before them.  Adjoint programs alternate between two buffers
-  // (pairs), so one barrier per exchange suffices: the previous reader of a
-  // buffer finished before the intervening exchange's barrier (or the barriers
-  // at the top of the tile loop).  A folded permutation run (t.fold) moves every amplitude from its
+  // Each state is written in the current layout and read back in the new one
+  // through its tile's one buffer (psi and lambda cross together, under one
+  // barrier); the ordering check below adds a block barrier before the writes
+  // when the previous exchange's readers are not ordered before them.
+  // A folded permutation run (t.fold) moves every amplitude from its
   // storage position x to F x ^ c on the way: the writes go to the permuted
   // positions, the reads are those of the new layout.
   const TFold* F = t.fold && folds_ ? &folds_[t.fold - 1] : nullptr;
@@ -552,12 +544,6 @@ void SegGen::emit_layout(const TOp& t) {
       if (F->omask[j]) o_ << " ^ ((0u - lqs::jit::obit(base, " << (int)F->oq[j] << ")) & " << hex32(F->omask[j]) << ")";
     o_ << ";\n";
   }
-  std::string jo;
-  if (adj_) {
-    jo = fresh("jo");
-    o_ << "    const uint32_t " << jo << " = " << swz_expr(wj, xs) << ";\n";
-  }
-  bool first = true;
   // who writes and who reads each buffer position in this exchange (with the
   // fold, for a tile whose outside bits are 0; a folded exchange is fenced by
   // block barriers, which hold for every tile)
@@ -566,100 +552,48 @@ void SegGen::emit_layout(const TOp& t) {
   wfold_ = nullptr;
   set_layout(t.ecmask);
   const std::vector<uint8_t> rown = owners(xs);
-  std::copy(saved_slot, saved_slot + 4, slot_);
+  std::copy(saved_slot, saved_slot + 4, slot_);  // barrier groups compare with the current layout
   std::copy(saved_thr, saved_thr + 16, thr_);
-  if (xpair_) {
-    // both states: writes into the pair, one barrier, reads from the pair.
-    // The pair used two exchanges ago was last read before the previous
-    // exchange's barrier.
-    const int bp = 2 * xp_, bl = 2 * xp_ + 1;
-    const char* XP = xp_ ? "XC" : "XA";
-    const char* XL = xp_ ? "XD" : "XB";
-    xp_ ^= 1;
-    bool unsafe = !exchange_safe(bp, wown) || !exchange_safe(bl, wown);
-    if (F)
-      for (const XRec& h : xhist_) unsafe = unsafe || ((h.bufs >> bp) & 1u) || ((h.bufs >> bl) & 1u);
-    if (unsafe) {
-      o_ << "    __syncthreads();  // earlier users of these buffers are not ordered before these writes\n";
-      next_bar_ = 1;
-      xhist_.clear();
-    }
-    uint32_t gmask = 0;
-    std::string bar;
-    if (F) {
-      bar = "__syncthreads();";
-      next_bar_ = 1;
-    } else {
-      bar = barrier_for(t.ecmask, &gmask);
-    }
-    if (!gmask) xhist_.clear();
-    xhist_.push_back(XRec{(1u << bp) | (1u << bl), gmask != 0, wown, rown, gmask});
-    o_ << "    { const uint32_t sj = " << jo << ";\n";
-    for (const char* pf : {"v", "u"}) {
-      pfx_ = pf;
-      for (int e = 0; e < R_; ++e) {
-        const uint32_t pos = F ? fold_lin(*F, old_je[e]) : old_je[e];
-        o_ << "      lqs::st_w(&" << (pf[0] == 'v' ? XP : XL) << "[" << xacc(xs, pos) << "], " << V(e) << ");\n";
-      }
-    }
-    pfx_ = "v";
-    o_ << "    }\n    " << bar << "\n";
-    set_layout(t.ecmask);  // validated by the caller
-    o_ << "    jt = " << jt_expr() << ";\n";
-    o_ << "    { const uint32_t sj = " << swz_expr("jt", xs) << ";\n";
-    for (const char* pf : {"v", "u"})
-      for (int e = 0; e < R_; ++e)
-        o_ << "      " << pf << e << " = lqs::ld_w(&" << (pf[0] == 'v' ? XP : XL) << "[" << xacc(xs, je(e)) << "]);\n";
-    o_ << "    }\n";
-    for (int e = 0; e < R_; ++e) vm_[e] = e;
-    if (t.e0 != t.ecmask) {
-      set_layout(t.e0);
-      o_ << "    jt = " << jt_expr() << ";\n";
-    }
-    return;
-  }
-  each([&]() {
-    const int xi = xb_;
-    const char* X = xb_ ? "XB" : "XA";
-    if (adj_) xb_ ^= 1;  // forward: the tile's one buffer
-    std::copy(saved_slot, saved_slot + 4, slot_);  // barrier groups compare with the current layout
-    std::copy(saved_thr, saved_thr + 16, thr_);
-    bool unsafe = !exchange_safe(xi, wown);
+  const int nst = adj_ ? 2 : 1;
+  bool unsafe = false;
+  for (int s = 0; s < nst; ++s) {
+    unsafe = unsafe || !exchange_safe(s, wown);
     if (F)  // the write positions move with each tile's outside bits: no earlier user of the buffer may be pending
-      for (const XRec& h : xhist_) unsafe = unsafe || ((h.bufs >> xi) & 1u);
-    if (unsafe) {
-      // a warp of another group may still use this buffer's positions from
-      // an earlier exchange: wait for the whole block first
-      o_ << "    __syncthreads();  // earlier users of this buffer are not ordered before these writes\n";
-      next_bar_ = 1;
-      xhist_.clear();
-    }
-    uint32_t gmask = 0;
-    std::string bar;
-    if (F) {
-      bar = "__syncthreads();";
-      next_bar_ = 1;
-    } else {
-      bar = barrier_for(t.ecmask, &gmask);
-    }
-    if (!gmask) xhist_.clear();
-    xhist_.push_back(XRec{1u << xi, gmask != 0, wown, rown, gmask});
-    if (adj_) o_ << "    { const uint32_t sj = " << jo << ";\n";
-    else o_ << "    { const uint32_t sj = " << swz_expr(wj, xs) << ";\n";
+      for (const XRec& h : xhist_) unsafe = unsafe || ((h.bufs >> s) & 1u);
+  }
+  if (unsafe) {
+    // a warp of another group may still use this buffer's positions from
+    // an earlier exchange: wait for the whole block first
+    o_ << "    __syncthreads();  // earlier users of this buffer are not ordered before these writes\n";
+    next_bar_ = 1;
+    xhist_.clear();
+  }
+  uint32_t gmask = 0;
+  std::string bar;
+  if (F) {
+    bar = "__syncthreads();";
+    next_bar_ = 1;
+  } else {
+    bar = barrier_for(t.ecmask, &gmask);
+  }
+  if (!gmask) xhist_.clear();
+  xhist_.push_back(XRec{nst == 2 ? 3u : 1u, gmask != 0, wown, rown, gmask});
+  o_ << "    { const uint32_t sj = " << swz_expr(wj, xs) << ";\n";
+  each([&]() {
     for (int e = 0; e < R_; ++e) {
       const uint32_t pos = F ? fold_lin(*F, old_je[e]) : old_je[e];
-      o_ << "      lqs::st_w(&" << X << "[" << xacc(xs, pos) << "], " << V(e) << ");\n";
+      o_ << "      lqs::st_w(&" << (pfx_[0] == 'v' ? "XA" : "XB") << "[" << xacc(xs, pos) << "], " << V(e) << ");\n";
     }
-    o_ << "    }\n    " << bar << "\n";
-    set_layout(t.ecmask);  // validated by the caller
-    if (first) o_ << "    jt = " << jt_expr() << ";\n";
-    first = false;
-    o_ << "    { const uint32_t sj = " << swz_expr("jt", xs) << ";\n";
-    for (int e = 0; e < R_; ++e)
-      o_ << "      " << pfx_ << e << " = lqs::ld_w(&" << X << "[" << xacc(xs, je(e)) << "]);\n";
-    o_ << "    }\n";
   });
-  if (!adj_) o_ << "@PF" << ++npf_ << "@";
+  o_ << "    }\n    " << bar << "\n";
+  set_layout(t.ecmask);  // validated by the caller
+  o_ << "    jt = " << jt_expr() << ";\n";
+  o_ << "    { const uint32_t sj = " << swz_expr("jt", xs) << ";\n";
+  each([&]() {
+    for (int e = 0; e < R_; ++e)
+      o_ << "      " << pfx_ << e << " = lqs::ld_w(&" << (pfx_[0] == 'v' ? "XA" : "XB") << "[" << xacc(xs, je(e)) << "]);\n";
+  });
+  o_ << "    }\n@PF" << ++npf_ << "@";
   for (int e = 0; e < R_; ++e) vm_[e] = e;
   if (t.e0 != t.ecmask) {  // relabelling SWAPs: from here on amplitudes carry their logical positions
     set_layout(t.e0);
@@ -1214,13 +1148,11 @@ bool SegGen::emit_op(const TOp& t) {
   }
 }
 
-// Forward segments run two CTAs per SM, each with one tile buffer: bulk loads
-// land in it, and once the tile is in registers the layout exchanges go
+// Kernels run two CTAs per SM, each with one buffer per tile: bulk loads land in it, and once the tile is in registers the layout exchanges go
 // through it.  After the last exchange has been read the buffer is free and
 // the next tile's load starts, behind the remaining ops and the stores of this
 // tile and the whole work of the other CTA.  FP32 pipe busy 57-68% against
-// 52-56% with one CTA per SM and a prefetch buffer (24-qubit ansatz); adjoint
-// sweeps hold two states and keep one CTA with separate exchange buffers.
+// 52-56% with one CTA per SM and a prefetch buffer (24-qubit ansatz).
 const char* kSkeletonHead = R"(
 extern "C" __global__ void __launch_bounds__(@NTH@, @MINB@)
 @NAME@(A::S* __restrict__ psi, @LAMP@const __grid_constant__ SegArgs P, @PARTP@int* status@FMTP@) {
@@ -1229,19 +1161,15 @@ extern "C" __global__ void __launch_bounds__(@NTH@, @MINB@)
   typedef A::C C;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const lqs::TileGeom& G = P.g;
-  S* S0 = reinterpret_cast<S*>(smem_raw);  // incoming tiles (bulk loads, prefetched one tile ahead)
-  S* S0L = S0 + @NT@;                      // incoming lambda tiles (adjoint only)
-  W* XA = reinterpret_cast<W*>(S0 + @NT@ * @NIN@);  // layout exchanges (forward: in the tile's own buffer)
-  W* XB = XA + @NT@;
-  W* XC = XB + @NT@;  // complex128 adjoint: the second pair of exchange buffers
-  W* XD = XC + @NT@;
-  double* wacc = reinterpret_cast<double*>(XA + @NT@ * @NX@);  // adjoint: per-warp gradient slots
+  S* S0 = reinterpret_cast<S*>(smem_raw);  // the tile (bulk loads)
+  S* S0L = S0 + @NT@;                      // the lambda tile (adjoint only)
+  W* XA = reinterpret_cast<W*>(S0);        // layout exchanges go through the tile's buffer
+  W* XB = reinterpret_cast<W*>(S0L);
+  double* wacc = reinterpret_cast<double*>(S0 + @NT@ * @NSTATES@);  // adjoint: per-warp gradient slots
   uint64_t* bar = reinterpret_cast<uint64_t*>(wacc + @NWACC@);
   const uint32_t tid = threadIdx.x;
   const uint32_t warp = tid >> 5;
-  (void)S0L;
-  (void)XC;
-  (void)XD;
+  (void)XB;
   (void)warp;
   for (uint32_t i = tid; i < @NWACC@; i += blockDim.x) wacc[i] = 0.0;
   uint64_t t = blockIdx.x;
@@ -1351,15 +1279,7 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
     set_layout(logical);
     o_ << "    jt = " << jt_expr() << ";\n";
   }
-  if (adj_) {
-    o_ << "    __syncthreads();  // the incoming buffers are free: prefetch the next tile into them\n"
-          "    { const uint64_t tn = t + gridDim.x;\n"
-          "      if (tn < G.ntiles) {\n"
-          "        lqs::jit::seg_copy(G, S0, psi, lqs::tile_base(G, tn), bar, my_roff);\n"
-          "        lqs::jit::seg_copy(G, S0L, lam, lqs::tile_base(G, tn), bar, my_roff);\n      } }\n";
-  } else {
-    o_ << "    __syncthreads();  // the tile has been read: its buffer serves the exchanges\n@PF0@";
-  }
+  o_ << "    __syncthreads();  // the tile has been read: its buffer serves the exchanges\n@PF0@";
   for (int i = first; i < nops; ++i) {
     if (ops[i].kind == K_LAYOUT) {
       if (i == nops - 1 && !ops[i].fold) {
@@ -1437,14 +1357,14 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
     fill(pre_, "t", "0u", "  ");
   }
   std::string body = replace_all(o_.str(), "@OFCUR@", "(phase ^ 1u) * " + std::to_string(ofac_.size()) + "u");
-  if (!adj_) {
-    // the next tile's load starts once the last exchange has been read
-    for (int i = 0; i < npf_; ++i) body = replace_all(body, "@PF" + std::to_string(i) + "@", "");
-    body = replace_all(body, "@PF" + std::to_string(npf_) + "@",
-                       std::string(npf_ ? "    lqs::fence_proxy_async();\n    __syncthreads();  // the buffer is free\n" : "") +
-                           "    { const uint64_t tn = t + gridDim.x;\n"
-                           "      if (tn < G.ntiles) lqs::jit::seg_copy(G, S0, psi, lqs::tile_base(G, tn), bar, my_roff); }\n");
-  }
+  // the next tile's load starts once the last exchange has been read
+  for (int i = 0; i < npf_; ++i) body = replace_all(body, "@PF" + std::to_string(i) + "@", "");
+  std::string pf = npf_ ? "    lqs::fence_proxy_async();\n    __syncthreads();  // the buffer is free\n" : "";
+  pf += "    { const uint64_t tn = t + gridDim.x;\n      if (tn < G.ntiles) {\n"
+        "        lqs::jit::seg_copy(G, S0, psi, lqs::tile_base(G, tn), bar, my_roff);\n";
+  if (adj_) pf += "        lqs::jit::seg_copy(G, S0L, lam, lqs::tile_base(G, tn), bar, my_roff);\n";
+  pf += "      } }\n";
+  body = replace_all(body, "@PF" + std::to_string(npf_) + "@", pf);
   const uint64_t h = fnv1a(body) ^ (fnv1a(pre_.str()) * 31u) ^ ((uint64_t)ncoef << 48) ^ ((uint64_t)k_ << 40) ^
                      ((uint64_t)b_ << 36) ^ ((uint64_t)ngrad << 24) ^ (adj_ ? 0x5a5aull : 0ull) ^ fnv1a(aname_);
   char nm[40];
@@ -1463,17 +1383,14 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
   s << "};\n";
   std::string head = replace_all(kSkeletonHead, "@NAME@", kname);
   head = replace_all(head, "@NTH@", std::to_string(nth));
-  // resident CTAs per SM the register budget aims at: forward two (1024 threads
-  // per SM with 128 bytes of state per thread, 512 with 256); adjoint 3 x 128, with 256 threads 2 (4 amplitudes of each state
-  // per thread) or 1 (8 or more), with 512 threads 1
-  const int minb = !adj_ ? std::max(1, (R_ * sz_ <= 128 ? 1024 : 512) / nth) : nth <= 128 ? 3 : nth >= 512 ? 1 : (R_ * sz_ <= 64 ? 2 : 1);
+  // resident CTAs per SM the register budget aims at: two (1024 threads per SM
+  // with 128 bytes of states per thread, 512 with 256)
+  const int minb = std::max(1, (R_ * sz_ * (adj_ ? 2 : 1) <= 128 ? 1024 : 512) / nth);
   head = replace_all(head, "@MINB@", std::to_string(minb));
   head = replace_all(head, "@LAMP@", adj_ ? "A::S* __restrict__ lam, " : "");
   head = replace_all(head, "@PARTP@", adj_ ? "double* partial, " : "");
   head = replace_all(head, "@FMTP@", ", const unsigned fmt");
   head = replace_all(head, "@NT@", std::to_string(1u << k_) + "u");
-  head = replace_all(head, "@NIN@", adj_ ? "2u" : "0u");
-  head = replace_all(head, "@NX@", xpair_ ? "4u" : adj_ ? "2u" : "1u");
   head = replace_all(head, "@NSTATES@", adj_ ? "2u" : "1u");
   head = replace_all(head, "@NWACC@", std::to_string(adj_ ? nwarps * kMaxGradSlotsJit : 0) + "u");
   head = replace_all(head, "@LAMCOPY0@",
@@ -2032,8 +1949,7 @@ int jit_adjoint_entry(const TileProg<A>& P, int r, void** entry, std::string* wh
 
 size_t jit_adjoint_smem(int k, int r, size_t amp_bytes) {
   const int warps = (1 << (k - r)) / 32;
-  const size_t tiles = amp_bytes == 16 ? 6 : 4;  // incoming psi and lambda, two (complex128: four) exchange buffers
-  return tiles * (amp_bytes << k) + sizeof(double) * warps * kMaxGradSlotsJit + 16;
+  return 2 * (amp_bytes << k) + sizeof(double) * warps * kMaxGradSlotsJit + 16;
 }
 
 template <class A>

@@ -72,3 +72,31 @@ def test_small_state_is_one_tile():
     c = W.ansatz(6, 3, 1)
     nseg, masks, _, _ = planned_order(c)
     assert nseg == 1 and masks[0] == (1 << 6) - 1
+
+
+@pytest.mark.parametrize("name,n,dtype", [("ansatz", 15, "c128"), ("ansatz", 16, "c64"), ("qft", 15, "c128"),
+                                          ("universal", 15, "c128"), ("random", 15, "c128"), ("random", 16, "c64")])
+def test_searched_plans_reproduce_the_circuit(name, n, dtype):
+    """Plans of compiled segments look for fuller tiles and let ops pass each other on wires that both leave in the
+    Z basis: the planned order must still give the in-order state, every non-diagonal target must sit in its
+    segment's tile, and no searched plan may need more passes than program order does."""
+    if name == "random":
+        names = [g for g, _, _ in W.GATES if g != "DoubleExcitation"]
+        c = W.random_circuit(n, 120, seed=7, names=names)
+    else:
+        c = W.ansatz(n, 4, 3) if name == "ansatz" else getattr(W, name)(n)
+    psi0 = W.gaussian_state(n, 5)
+    old = L.lqs_jit_info()["mode"]
+    try:
+        L.lqs_set_jit(L.LQS_JIT_ON)
+        nseg, masks, seg_of, order = planned_order(c, None, dtype)
+        L.lqs_set_jit(L.LQS_JIT_OFF)  # no compiled kernels, no dense cap: program order
+        plain = planned_order(c, {"max_ops": 16}, dtype)[0]
+    finally:
+        L.lqs_set_jit(old)
+    np.testing.assert_allclose(run_in_order(c, order, psi0), oracle.run_circuit(c, psi0), atol=1e-12)
+    for i, op in enumerate(c.ops):
+        if op.name not in DIAG and op.name not in ("U2", "U4"):
+            targets = op.wires[-2:] if op.name in ("SWAP", "CSWAP") else op.wires[-1:]
+            assert all((masks[seg_of[i]] >> t) & 1 for t in targets), (op.name, op.wires)
+    assert nseg <= plain
