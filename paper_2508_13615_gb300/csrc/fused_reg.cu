@@ -69,6 +69,17 @@ int reg_tile_qubits(int dtype) { return (dtype == LQS_C64 ? 4 : 3) + kRegThreadB
 #endif
 template <class A> struct JitR { static constexpr int r = LQS_SEG_RBITS_C128; };
 template <> struct JitR<ArF32> { static constexpr int r = 4; };
+// Complex128 segments with dense complex gates keep 3: twice the amplitudes
+// per thread doubled code that is long already, and a segment of four-by-four
+// updates took NVRTC 45 s instead of 10 (90 random gates on 14 qubits).
+template <class A>
+static int jit_rbits(const std::vector<KOp>& ops, const Segment& seg) {
+  int r = JitR<A>::r;
+  if (A::kAmpBytes == 16)
+    for (int i : seg.ops)
+      if (ops[i].kind == K_DENSE1 || ops[i].kind == K_DENSE2) r = std::min(r, 3);
+  return r;
+}
 
 // ---------------------------------------------------------------------------
 // device side
@@ -804,7 +815,7 @@ template <class A>
 int launch_fused_reg_t(SV* sv, const std::vector<KOp>& ops, const Segment& seg, int k, int b, int arith,
                        unsigned fmt) {
   constexpr int R = RegR<A>::R;
-  const int r = RLog<R>::r, rj = JitR<A>::r;
+  const int r = RLog<R>::r, rj = jit_rbits<A>(ops, seg);
   static thread_local TileProg<A> P;
   init_prog(P, sv->n, seg.qmask, k, b);
   const bool jit = jit_enabled_for(sv->n);  // compiled segments fold permutation runs into exchanges
@@ -848,8 +859,9 @@ static int note_reg_prog_t(int n, const std::vector<KOp>& ops, const Segment& se
   constexpr int R = RegR<A>::R;
   static thread_local TileProg<A> P;
   init_prog(P, n, seg.qmask, k, b);
-  LQS_TRY(build_reg_prog(P, ops, seg, JitR<A>::r, nullptr, true));
-  return jit_note(P, JitR<A>::r, n, force, todo);
+  const int r = jit_rbits<A>(ops, seg);
+  LQS_TRY(build_reg_prog(P, ops, seg, r, nullptr, true));
+  return jit_note(P, r, n, force, todo);
 }
 
 int note_reg_prog(int n, int dtype, int arith, const std::vector<KOp>& ops, const Segment& seg, int k, int b,
@@ -1052,8 +1064,9 @@ bool seg_split_capable(const SV* sv, const std::vector<KOp>& ops, const Segment&
   if (k != reg_tile_qubits(sv->dtype) || !jit_enabled_for(sv->n)) return false;
   static thread_local TileProg<ArDF> P;
   init_prog(P, sv->n, seg.qmask, k, b);
-  if (build_reg_prog(P, ops, seg, JitR<ArDF>::r, nullptr, true) != LQS_OK) return false;  // launched split in two
-  return jit_ready(P, JitR<ArDF>::r, sv);
+  const int r = jit_rbits<ArDF>(ops, seg);
+  if (build_reg_prog(P, ops, seg, r, nullptr, true) != LQS_OK) return false;  // launched split in two
+  return jit_ready(P, r, sv);
 }
 
 }  // namespace lqs
