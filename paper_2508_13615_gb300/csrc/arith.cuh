@@ -203,11 +203,17 @@ LQS_HD DF df_sub(DF a, DF b) { return df_add(a, df_neg(b)); }
 // straight-line code: 48 double-float rotations of 8 amplitudes (147 KB of
 // scalar instructions) ran at 25 T operations/s, the packed form at 31 T, and
 // up to 24 rotations (37 KB packed) at 39.5 T, the full float32 rate.
+//
+// Packing is volatile for the compiler's sake: as plain values the chains of
+// packing and unpacking in a long segment cost the optimiser time superlinear
+// in the code.  A reverse segment of RX gates on 24 qubits took 155 s to build,
+// and takes 6 s; one of RY and RZ gates 10 and 4 s.  Registers, spills and code
+// size are the same.
 #ifdef __CUDACC__
 typedef unsigned long long f2;
 __device__ __forceinline__ f2 f2_pack(float lo, float hi) {
   f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  asm volatile("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
   return r;
 }
 __device__ __forceinline__ void f2_unpack(f2 a, float& lo, float& hi) {

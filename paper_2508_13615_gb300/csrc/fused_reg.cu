@@ -69,9 +69,13 @@ int reg_tile_qubits(int dtype) { return (dtype == LQS_C64 ? 4 : 3) + kRegThreadB
 #endif
 template <class A> struct JitR { static constexpr int r = LQS_SEG_RBITS_C128; };
 template <> struct JitR<ArF32> { static constexpr int r = 4; };
-// Complex128 segments with dense complex gates keep 3: twice the amplitudes
-// per thread doubled code that is long already, and a segment of four-by-four
-// updates took NVRTC 45 s instead of 10 (90 random gates on 14 qubits).
+// Complex128 segments with dense complex gates keep 3 (512 threads, two CTAs
+// per SM at 64 registers each): their code is long, and twice the amplitudes
+// per thread double it.  24 qubits, 3 bits / 4 bits / 3 bits with one CTA per SM
+// and 128 registers: 4 layers RX + RZ 5.07 / 5.65 / 5.26 ms, Rot 4.59 / 4.94 /
+// 4.83, U4 windows 4.46 / 4.64 / 4.56, U4 brick 4.87 / 5.07 / 5.03, 200 random
+// gates 7.73 / 8.08 / 8.20.  The spills of 64 registers (up to 400 bytes) cost
+// less than what the second CTA hides.
 template <class A>
 static int jit_rbits(const std::vector<KOp>& ops, const Segment& seg) {
   int r = JitR<A>::r;

@@ -112,39 +112,25 @@ template <> struct Lz<ArDFP> {
     return A;
   }
   static __device__ __forceinline__ W cmul(const DFK& c, const W& a) { return p2_raw(cprod(k2(c), a)); }
-  // Dense complex rows in scalar form: packed ones need every coefficient's
-  // parts in pairs, and the code took the compiler 20 times as long.
-  static __device__ __forceinline__ void row(DAcc& re, DAcc& im, const DFK& c, const W& w) {
-    DF x, y;
-    p2_lanes(w, x, y);
-    df_mac(re, x, c.re);
-    df_mac(re, df_neg(y), c.im);
-    df_mac(im, y, c.re);
-    df_mac(im, x, c.im);
-  }
-  static __device__ __forceinline__ void row0(DAcc& re, DAcc& im, const DFK& c, const W& w) {
-    DF x, y;
-    p2_lanes(w, x, y);
-    re = df_prod(x, c.re);
-    df_mac(re, df_neg(y), c.im);
-    im = df_prod(y, c.re);
-    df_mac(im, x, c.im);
-  }
-  static __device__ __forceinline__ W pair(const DAcc& re, const DAcc& im) {
-    return W{f2_pack(re.s, im.s), f2_pack(re.e, im.e)};
+  // Dense complex rows, two packed products per coefficient: results are those
+  // of the scalar rows bit for bit, in half the instructions.  24 qubits, scalar
+  // against packed: reverse sweep of 4 layers RX + RZ 18.7 -> 14.7 ms, of 3 brick
+  // layers of U4 12.7 -> 9.4, forward 4 layers RX + RZ 6.4 -> 5.1, U4 windows
+  // 5.1 -> 4.5; a reverse segment of RX gates builds in 6 s instead of 13.
+  static __device__ __forceinline__ void cmac(PAcc& A, const K2& c, const W& a) {
+    p2_mac(A, a, c.c);
+    p2_mac(A, p2_swap(a), c.s);
   }
   static __device__ __forceinline__ W cmac2(const DFK& c0, const W& a, const DFK& c1, const W& b) {
-    DAcc re, im;
-    row0(re, im, c0, a);
-    row(re, im, c1, b);
-    return pair(re, im);
+    PAcc A = cprod(k2(c0), a);
+    cmac(A, k2(c1), b);
+    return p2_raw(A);
   }
   static __device__ __forceinline__ W cmac4(const DFK* c, const W* a) {
-    DAcc re, im;
-    row0(re, im, c[0], a[0]);
+    PAcc A = cprod(k2(c[0]), a[0]);
 #pragma unroll
-    for (int i = 1; i < 4; ++i) row(re, im, c[i], a[i]);
-    return pair(re, im);
+    for (int i = 1; i < 4; ++i) cmac(A, k2(c[i]), a[i]);
+    return p2_raw(A);
   }
   static __device__ __forceinline__ DFK kmul(const DFK& a, const DFK& b) {
     DFK r;

@@ -311,3 +311,27 @@ def test_permutation_runs_fold_into_exchanges(tmp_path, monkeypatch):
     assert not bad, bad
     races = {f: r[:3] for f in folded for r in [_unordered_accesses(open(f).read())] if r}
     assert not races, races
+
+
+def test_dense_complex_gates_build_about_as_fast_as_real_ones():
+    """Kernels of dense complex gates (RX) hold twice the multiplications of
+    real rotations (RY) and no more ops; the time to build one has to follow
+    that, not grow faster with the code: at most four times RY's, in the
+    reverse sweep (21 qubits) and forward (23)."""
+    def seconds_per_kernel(gate, n, adjoint):
+        c = W.Circuit(n)
+        for _ in range(2):
+            for name in (gate, "RZ"):
+                for q in range(n):
+                    c.add(name, (q,), (0.3 + 0.01 * q,))
+            for q in range(n - 1):
+                c.add("CNOT", (q, q + 1))
+        build = L.lqs_jit_precompile_adjoint if adjoint else L.lqs_jit_precompile
+        before = L.lqs_jit_info()["compile_seconds"]
+        built = build(n, "c128", c.ops, c.params, L.LQS_ARITH_DF)
+        assert built > 0
+        return (L.lqs_jit_info()["compile_seconds"] - before) / built
+
+    for n, adjoint in ((21, True), (23, False)):
+        real, dense = (seconds_per_kernel(g, n, adjoint) for g in ("RY", "RX"))
+        assert dense <= 4.0 * real, (adjoint, real, dense)
