@@ -21,14 +21,18 @@
 #include "tile_ops.cuh"
 
 // Dense work per segment: a compiled segment is straight-line code, and one
-// whose dense updates add up past this weight (4 per two-qubit dense op, 1
+// whose dense updates add up past this weight (3 per two-qubit dense op, 1
 // per one-qubit dense op; diagonal and permutation ops are free) spends more
 // in instruction fetch than a further pass costs.  30-qubit 10-layer ansatz,
 // complex128: caps of 8 / 12 / 16 / 24 / 40 ran 451 / 418 / 426 / 453 / 510 ms.
+// Two-qubit ops weigh 3, so that a segment takes four: with 4 (three to a
+// segment) U4 windows on 24 qubits ran 4.46 ms, a U4 brick circuit 4.87, 200
+// random gates 7.75; with 3 4.34, 4.74, 7.54.
 #ifndef LQS_SEGMENT_DENSE_CAP
 #define LQS_SEGMENT_DENSE_CAP 12
 #endif
-// complex64 segments carry float32 arithmetic, several times less code per op
+// complex64 segments carry float32 arithmetic, several times less code per op;
+// their two-qubit ops weigh 4
 #ifndef LQS_SEGMENT_DENSE_CAP_C64
 #define LQS_SEGMENT_DENSE_CAP_C64 64
 #endif
@@ -47,6 +51,7 @@ int resolve_cfg(int n, int dtype, const lqs_fuse_cfg* cfg, PlanCfg& pc, int* ari
   pc.dense_cap = n > reg_tile_qubits(dtype) && jit_enabled_for(n)
                      ? (dtype == LQS_C64 ? LQS_SEGMENT_DENSE_CAP_C64 : LQS_SEGMENT_DENSE_CAP)
                      : 0;
+  if (dtype == LQS_C64) pc.dense2_weight = 4;
   int ar = LQS_ARITH_AUTO;
   if (cfg) {
     if (cfg->tile_qubits) pc.k = cfg->tile_qubits;
@@ -97,8 +102,8 @@ static int coef_count(const KOp& o) {
 // Diagonal ops and controls need no tile qubit.  Ops on disjoint wires
 // commute; searched plans also let ops pass each other when every wire they
 // share is one that both leave in the Z basis (controls, diagonal targets).
-static int dense_weight(const KOp& o) {
-  return o.kind == K_DENSE2 ? 4 : (o.kind == K_DENSE1 || o.kind == K_DENSE1R) ? 1 : 0;
+static int dense_weight(const KOp& o, int w2) {
+  return o.kind == K_DENSE2 ? w2 : (o.kind == K_DENSE1 || o.kind == K_DENSE1R) ? 1 : 0;
 }
 
 
@@ -208,7 +213,7 @@ int plan_segments(int n, const std::vector<KOp>& ops, const PlanCfg& pc, std::ve
   auto set_pass = [&](bool commute) {
     for (size_t i = 0; i < ops.size(); ++i) {
       const uint64_t t = ops[i].tile_mask(), w = ops[i].wire_mask();
-      po[i] = POp{commute ? t : w, commute ? w & ~t : 0, t, coef_count(ops[i]), dense_weight(ops[i])};
+      po[i] = POp{commute ? t : w, commute ? w & ~t : 0, t, coef_count(ops[i]), dense_weight(ops[i], pc.dense2_weight)};
     }
   };
   set_pass(false);

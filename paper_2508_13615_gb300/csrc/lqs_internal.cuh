@@ -135,6 +135,7 @@ struct PlanCfg {
   int b = 0;          // low contiguous qubits
   int max_ops = 0;    // per-segment cap
   int dense_cap = 0;  // cap on a segment's dense weight (compiled segments; 0 = none)
+  int dense2_weight = 3;  // of a two-qubit dense op (a one-qubit one weighs 1)
   bool search = false;  // look for tiles that execute more per pass (compiled complex128 segments)
 };
 int resolve_cfg(int n, int dtype, const lqs_fuse_cfg* cfg, PlanCfg& pc, int* arith);

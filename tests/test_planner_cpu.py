@@ -100,3 +100,18 @@ def test_searched_plans_reproduce_the_circuit(name, n, dtype):
             targets = op.wires[-2:] if op.name in ("SWAP", "CSWAP") else op.wires[-1:]
             assert all((masks[seg_of[i]] >> t) & 1 for t in targets), (op.name, op.wires)
     assert nseg <= plain
+
+
+def test_four_two_qubit_gates_share_a_compiled_segment():
+    """The cap on a compiled complex128 segment's dense work leaves room for four two-qubit matrices: eight of them in
+    one tile take two passes."""
+    n = 14
+    c = W.Circuit(n)
+    for i in range(8):
+        c.add("U4", (i % 5, 5 + i % 4), matrix=W.haar_unitary(4, i))
+    old = L.lqs_jit_info()["mode"]
+    try:
+        L.lqs_set_jit(L.LQS_JIT_ON)
+        assert L.lqs_plan_fused(n, "c128", c.ops, None)[0] == 2
+    finally:
+        L.lqs_set_jit(old)
