@@ -645,7 +645,7 @@ int lqs_jit_precompile_adjoint(int n_qubits, int dtype, int arith, const lqs_op*
   rev.reserve(kops.size());
   for (size_t i = kops.size(); i-- > 0;) rev.push_back(inverse_op(kops[i]));
   const int ar = current_arith(arith);
-  if (n_qubits <= adjoint_tile_qubits(dtype)) return LQS_OK;  // one tile: the interpreter sweep runs it
+  if (n_qubits <= adjoint_tile_qubits()) return LQS_OK;  // one tile: the interpreter sweep runs it
   return adjoint_precompile(n_qubits, dtype, ar, rev, n_compiled);
 }
 
@@ -661,7 +661,12 @@ int lqs_jit_precompile(int n_qubits, int dtype, int arith, const lqs_op* ops, in
   PlanCfg pc;
   int ar = LQS_ARITH_AUTO;
   LQS_TRY(resolve_cfg(n_qubits, dtype, cfg, pc, &ar));
-  if (arith != LQS_ARITH_AUTO) ar = arith;
+  if (arith != LQS_ARITH_AUTO && arith != ar) {  // the plan depends on the arithmetic too
+    lqs_fuse_cfg c = cfg ? *cfg : lqs_fuse_cfg{};
+    c.arith = arith;
+    pc = PlanCfg{};
+    LQS_TRY(resolve_cfg(n_qubits, dtype, &c, pc, &ar));
+  }
   std::vector<Segment> segs;
   LQS_TRY(plan_segments(n_qubits, kops, pc, segs));
   std::vector<void*> todo;

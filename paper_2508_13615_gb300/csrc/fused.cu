@@ -36,6 +36,14 @@
 #ifndef LQS_SEGMENT_DENSE_CAP_C64
 #define LQS_SEGMENT_DENSE_CAP_C64 64
 #endif
+// The float64 policy is bound by its pipe, not by instruction fetch: caps of
+// 12 / 16 / 24 ran 24-qubit circuits of 4 layers RX + RZ in 28.6 / 28.7 / 28.2 ms,
+// U4 windows 32.7 / 32.6 / 32.4, a 10-layer ansatz 26.7 / 27.2 / 26.3.  Searched
+// plans helped the ansatz (25.0 ms) and cost the universal circuit 18% (18.6 ->
+// 21.9): fewer passes, more diagonal products.
+#ifndef LQS_SEGMENT_DENSE_CAP_F64
+#define LQS_SEGMENT_DENSE_CAP_F64 24
+#endif
 
 namespace lqs {
 
@@ -47,10 +55,6 @@ int resolve_cfg(int n, int dtype, const lqs_fuse_cfg* cfg, PlanCfg& pc, int* ari
   pc.k = reg_tile_qubits(dtype);                  // the register-tile kernel's shape
   pc.b = dtype == LQS_C64 ? 5 : 4;
   pc.max_ops = kMaxTileOps;
-  // multi-tile states whose segments run as compiled code
-  pc.dense_cap = n > reg_tile_qubits(dtype) && jit_enabled_for(n)
-                     ? (dtype == LQS_C64 ? LQS_SEGMENT_DENSE_CAP_C64 : LQS_SEGMENT_DENSE_CAP)
-                     : 0;
   if (dtype == LQS_C64) pc.dense2_weight = 4;
   int ar = LQS_ARITH_AUTO;
   if (cfg) {
@@ -67,15 +71,22 @@ int resolve_cfg(int n, int dtype, const lqs_fuse_cfg* cfg, PlanCfg& pc, int* ari
   if (pc.b < std::max(bmin, 1) || pc.b > pc.k - 2)
     return set_error(LQS_ERR_ARG, "low_qubits must be in [1, tile_qubits - 2]");
   if (pc.max_ops < 1) return set_error(LQS_ERR_ARG, "max_ops must be positive");
+  ar = current_arith(ar);
+  const bool f64 = dtype == LQS_C128 && ar == LQS_ARITH_F64;
+  // multi-tile states whose segments run as compiled code
+  if (n > reg_tile_qubits(dtype) && jit_enabled_for(n))
+    pc.dense_cap = dtype == LQS_C64 ? LQS_SEGMENT_DENSE_CAP_C64 : f64 ? LQS_SEGMENT_DENSE_CAP_F64 : LQS_SEGMENT_DENSE_CAP;
   // complex128 only: another order of commuting gates rounds differently, far
   // below double precision but by up to the last float32 bit in complex64,
-  // whose energies and gradients are to stay what program order gives
-  pc.search = dtype == LQS_C128 && pc.dense_cap > 0 && pc.k == reg_tile_qubits(dtype);
+  // whose energies and gradients are to stay what program order gives.  Not for
+  // the float64 policy either: its float64 pipe is the bound, and searched plans
+  // trade passes for more diagonal products (LQS_SEGMENT_DENSE_CAP_F64)
+  pc.search = dtype == LQS_C128 && !f64 && pc.dense_cap > 0 && pc.k == reg_tile_qubits(dtype);
   if (n <= pc.k) {  // the whole state is one tile
     pc.k = n;
     pc.b = n;
   }
-  if (arith) *arith = current_arith(ar);
+  if (arith) *arith = ar;
   return LQS_OK;
 }
 

@@ -75,7 +75,8 @@ template <> struct JitR<ArF32> { static constexpr int r = 4; };
 // and 128 registers: 4 layers RX + RZ 5.07 / 5.65 / 5.26 ms, Rot 4.59 / 4.94 /
 // 4.83, U4 windows 4.46 / 4.64 / 4.56, U4 brick 4.87 / 5.07 / 5.03, 200 random
 // gates 7.73 / 8.08 / 8.20.  The spills of 64 registers (up to 400 bytes) cost
-// less than what the second CTA hides.
+// less than what the second CTA hides.  In the float64 policy they do not (its
+// pipe is busy with one CTA): those segments have an SM to themselves.
 template <class A>
 static int jit_rbits(const std::vector<KOp>& ops, const Segment& seg) {
   int r = JitR<A>::r;
@@ -879,13 +880,16 @@ int note_reg_prog(int n, int dtype, int arith, const std::vector<KOp>& ops, cons
 // compiled adjoint (reverse sweep over psi and lambda)
 // ---------------------------------------------------------------------------
 // The kernel holds a tile of 2^11 amplitudes of psi and of lambda in
-// registers: complex128 in 256 threads (8 of each state per thread), complex64
-// in 128 (16 per thread), one buffer per tile, two and four CTAs per SM.
-static void adj_shape(int dtype, int* r, int* tb) {
-  *r = dtype == LQS_C64 ? 4 : 3;
-  *tb = dtype == LQS_C64 ? 7 : 8;
-}
-// Dense work per reverse segment (complex128): an op costs about four times
+// registers, one buffer per tile.  Register bits per state: complex64 4 (128
+// threads, four CTAs per SM), double-float 3 (256 threads, two), float64 2 (512
+// threads, one: 8 amplitudes per thread spill up to 1 KB, and the float64 pipe
+// is the bound at any occupancy; 24 qubits, 3 bits against 2: RX + RY 82.2 and
+// 80.4 ms, RX 56.2 and 54.6, RX + RZ 62.8 and 61.5).
+constexpr int kAdjTileQubits = 11;
+template <class A> struct AdjR { static constexpr int r = 3; };
+template <> struct AdjR<ArF64> { static constexpr int r = 2; };
+template <> struct AdjR<ArF32> { static constexpr int r = 4; };
+// Dense work per reverse segment (double-float): an op costs about four times
 // its forward code (two states and a partial), and the search for fuller
 // segments makes them longer than the instruction cache holds.  24-qubit
 // 8-layer gradient: 45 ms without a cap (25 ms with the program-order plan);
@@ -894,14 +898,10 @@ static void adj_shape(int dtype, int* r, int* tb) {
 #ifndef LQS_ADJOINT_DENSE_CAP
 #define LQS_ADJOINT_DENSE_CAP 16
 #endif
-int adjoint_tile_qubits(int dtype) {
-  int r, tb;
-  adj_shape(dtype, &r, &tb);
-  return r + tb;
-}
+int adjoint_tile_qubits() { return kAdjTileQubits; }
 
 bool reg_adjoint_available(const SV* sv, int) {
-  return jit_enabled_for(sv->n) && sv->n > adjoint_tile_qubits(sv->dtype);
+  return jit_enabled_for(sv->n) && sv->n > kAdjTileQubits;
 }
 
 template <class A>
@@ -939,15 +939,13 @@ static int adj_build(int n, const std::vector<KOp>& rev, const Segment& seg, int
 template <class A>
 static int adj_prepare_t(int n, int dtype, const std::vector<KOp>& rev, std::vector<std::unique_ptr<AdjProg<A>>>& progs,
                          int* compiled, bool force) {
-  int r, tb;
-  adj_shape(dtype, &r, &tb);
-  const int k = r + tb, b = dtype == LQS_C64 ? 5 : 4;
+  const int r = AdjR<A>::r, k = kAdjTileQubits, b = dtype == LQS_C64 ? 5 : 4;
   if (n <= k) return set_error(LQS_ERR_UNSUPPORTED, "state fits one adjoint tile");
   PlanCfg pc;
   pc.k = k;
   pc.b = b;
   pc.max_ops = kMaxTileOps;
-  if (dtype == LQS_C128) {  // complex64 keeps program order (resolve_cfg)
+  if (std::is_same<A, ArDF>::value) {  // the others keep program order (resolve_cfg)
     pc.search = true;
     pc.dense_cap = LQS_ADJOINT_DENSE_CAP;
   }
@@ -977,9 +975,7 @@ template <class A>
 static int run_adjoint_compiled_t(SV* sv, const std::vector<KOp>& rev, void* lam, int arith,
                                   std::vector<int>& slot_op, std::vector<double>& slot_scale, double** partial_out,
                                   int* grid_out) {
-  int r, tb;
-  adj_shape(sv->dtype, &r, &tb);
-  const int n = sv->n, k = r + tb;
+  const int n = sv->n, r = AdjR<A>::r, k = kAdjTileQubits;
   std::vector<std::unique_ptr<AdjProg<A>>> progs;
   LQS_TRY(adj_prepare_t<A>(n, sv->dtype, rev, progs, nullptr, false));
   size_t nslots = 0;

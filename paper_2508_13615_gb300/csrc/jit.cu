@@ -1384,8 +1384,11 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
   std::string head = replace_all(kSkeletonHead, "@NAME@", kname);
   head = replace_all(head, "@NTH@", std::to_string(nth));
   // resident CTAs per SM the register budget aims at: two (1024 threads per SM
-  // with 128 bytes of states per thread, 512 with 256)
-  const int minb = std::max(1, (R_ * sz_ * (adj_ ? 2 : 1) <= 128 ? 1024 : 512) / nth);
+  // with 128 bytes of states per thread, 512 with 256), one for 512 threads of
+  // float64 (64 registers spill, and its pipe is busy anyway; 24 qubits, one
+  // against two: U4 windows 32.6 and 33.7 ms, RX + RZ 28.7 and 29.5)
+  const bool f64 = aname_ == std::string("lqs::ArF64");
+  const int minb = f64 && nth >= 512 ? 1 : std::max(1, (R_ * sz_ * (adj_ ? 2 : 1) <= 128 ? 1024 : 512) / nth);
   head = replace_all(head, "@MINB@", std::to_string(minb));
   head = replace_all(head, "@LAMP@", adj_ ? "A::S* __restrict__ lam, " : "");
   head = replace_all(head, "@PARTP@", adj_ ? "double* partial, " : "");

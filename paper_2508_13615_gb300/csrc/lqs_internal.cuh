@@ -169,7 +169,7 @@ bool seg_split_capable(const SV* sv, const std::vector<KOp>& ops, const Segment&
 // slot_scale: the factor each slot's summed partials take).  Returns
 // LQS_ERR_UNSUPPORTED, having launched nothing, when the interpreter must run.
 bool reg_adjoint_available(const SV* sv, int arith);
-int adjoint_tile_qubits(int dtype);  // tile of the compiled reverse sweep
+int adjoint_tile_qubits();  // tile of the compiled reverse sweep
 int run_adjoint_compiled(SV* sv, const std::vector<KOp>& rev, void* lam, int arith, std::vector<int>& slot_op,
                          std::vector<double>& slot_scale, double** partial, int* grid);
 // Host only: compile the reverse sweep's kernels (rev = inverse ops, reversed).

@@ -335,3 +335,24 @@ def test_dense_complex_gates_build_about_as_fast_as_real_ones():
     for n, adjoint in ((21, True), (23, False)):
         real, dense = (seconds_per_kernel(g, n, adjoint) for g in ("RY", "RX"))
         assert dense <= 4.0 * real, (adjoint, real, dense)
+
+
+def test_float64_reverse_sweep_keeps_its_states_in_registers(tmp_path, monkeypatch):
+    """The float64 reverse sweep holds 128 bytes of psi and lambda per thread;
+    its kernels spill at most twice that (temporaries of one op), as ptxas
+    reports it."""
+    import glob
+    import re
+    monkeypatch.setenv("LQS_JIT_DUMP", str(tmp_path))
+    n = 16
+    c = W.Circuit(n)
+    for _ in range(4):
+        for name in ("RX", "RZ"):
+            for q in range(n):
+                c.add(name, (q,), (0.2 + 0.01 * q,))
+        for q in range(n - 1):
+            c.add("CNOT", (q, q + 1))
+    assert L.lqs_jit_precompile_adjoint(n, "c128", c.ops, c.params, L.LQS_ARITH_F64) > 0
+    logs = "".join(open(f).read() for f in glob.glob(str(tmp_path / "lqs_adj_*.log")))
+    spills = [int(x) for x in re.findall(r"(\d+) bytes spill stores", logs)]
+    assert spills and max(spills) <= 256, spills

@@ -115,3 +115,47 @@ def test_four_two_qubit_gates_share_a_compiled_segment():
         assert L.lqs_plan_fused(n, "c128", c.ops, None)[0] == 2
     finally:
         L.lqs_set_jit(old)
+
+
+def program_order_passes(c, k, b, cap, w2):
+    """Passes of the plain greedy plan: a segment takes every op, in program order, that shares no wire with an op it
+    has left behind and whose non-diagonal targets fit the tile, up to 128 ops and the cap on dense work."""
+    dense = {"H": 1, "RX": 1, "RY": 1, "Rot": 1, "U2": 1, "CRY": 1, "U4": w2}
+    left, passes = list(range(len(c.ops))), 0
+    while left:
+        tile, blocked, work, taken, rest = set(range(b)), set(), 0, 0, []
+        for i in left:
+            op = c.ops[i]
+            t = set() if op.name in DIAG else set(op.wires[-2:] if op.name in ("SWAP", "CSWAP", "U4") else op.wires[-1:])
+            w = dense.get(op.name, 0)
+            if not (blocked & set(op.wires)) and len(tile | t) <= k and taken < 128 and (work + w <= cap or not taken):
+                tile, work, taken = tile | t, work + w, taken + 1
+            else:
+                blocked |= set(op.wires)
+                rest.append(i)
+        assert len(rest) < len(left)
+        left, passes = rest, passes + 1
+    return passes
+
+
+@pytest.mark.parametrize("name", ["ansatz", "qft", "universal", "random"])
+def test_searched_plans_against_program_order(name):
+    """Double-float plans of compiled segments never take more passes than program order under the same cap on dense
+    work, and fewer where layers overlap (ansatz, universal circuit).  The float64 policy and complex64 keep program
+    order: exactly its number of passes."""
+    n = 18
+    if name == "random":
+        c = W.random_circuit(n, 120, seed=7, names=[g for g, _, _ in W.GATES if g != "DoubleExcitation"])
+    else:
+        c = W.ansatz(n, 6, 3) if name == "ansatz" else getattr(W, name)(n)
+    old = L.lqs_jit_info()["mode"]
+    try:
+        L.lqs_set_jit(L.LQS_JIT_ON)
+        passes = {a: L.lqs_plan_fused(n, "c128", c.ops, {"arith": a})[0] for a in (L.LQS_ARITH_DF, L.LQS_ARITH_F64)}
+        c64 = L.lqs_plan_fused(n, "c64", c.ops, None)[0]
+    finally:
+        L.lqs_set_jit(old)
+    plain = program_order_passes(c, 12, 4, 12, 3)
+    assert passes[L.LQS_ARITH_DF] < plain if name in ("ansatz", "universal") else passes[L.LQS_ARITH_DF] <= plain
+    assert passes[L.LQS_ARITH_F64] == program_order_passes(c, 12, 4, 24, 3)
+    assert c64 == program_order_passes(c, 13, 5, 64, 4)
