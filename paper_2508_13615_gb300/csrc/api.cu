@@ -693,6 +693,7 @@ int lqs_plan_fused(int n_qubits, int dtype, const lqs_op* ops, int n_ops, const 
   // Map lowered ops back to the caller's ops: lower one op at a time.
   std::vector<KOp> kops;
   std::vector<int> owner;
+  kops.reserve((size_t)n_ops);
   for (int i = 0; i < n_ops; ++i) {
     const size_t before = kops.size();
     LQS_TRY(lower_ops(n_qubits, ops + i, 1, zeros.data(), (int)zeros.size(), false, kops));

@@ -6,6 +6,7 @@ CPU oracle must therefore reproduce the in-order result; and every segment's
 tile must hold the low qubits and every non-diagonal target of its gates.
 """
 import math
+import time
 
 import numpy as np
 import pytest
@@ -159,3 +160,30 @@ def test_searched_plans_against_program_order(name):
     assert passes[L.LQS_ARITH_DF] < plain if name in ("ansatz", "universal") else passes[L.LQS_ARITH_DF] <= plain
     assert passes[L.LQS_ARITH_F64] == program_order_passes(c, 12, 4, 24, 3)
     assert c64 == program_order_passes(c, 13, 5, 64, 4)
+
+
+def test_planning_time_is_proportional_to_the_circuit():
+    """Phase-estimation shape: one wire is never a target, so it never blocks.  Planning eight times the ops may take
+    twice its share of the time, far from the 64 of a search that scans the whole circuit for every segment."""
+    n = 30
+
+    def seconds(m, seed):
+        r = W.splitmix64(seed, 0, m)
+        c = W.Circuit(n)
+        c.params = np.array([0.3])
+        for i in range(m):
+            q = 1 + int(r[i] % np.uint64(n - 1))
+            c.ops.append([W.Op("RY", (q,), 0), W.Op("ControlledPhaseShift", (0, q), 0),
+                          W.Op("CNOT", (q, 1 + q % (n - 1)))][i % 3])
+        ops = L.OpArray(c.ops)
+        t0 = time.process_time()
+        L.lqs_plan_fused(n, "c128", ops, None)
+        return time.process_time() - t0
+
+    old = L.lqs_jit_info()["mode"]
+    try:
+        L.lqs_set_jit(L.LQS_JIT_ON)
+        small = min(seconds(4000, s) for s in (1, 2, 3))
+        assert seconds(32000, 4) <= 16 * small
+    finally:
+        L.lqs_set_jit(old)
