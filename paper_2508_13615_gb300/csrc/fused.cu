@@ -221,9 +221,11 @@ int make_plan(int n, const std::vector<POp>& ops, const PlanCfg& pc, bool search
 }
 
 // Plans with a search cost 2-20 ms of host time (300-900 ops), so they are
-// kept by structure: everything the plan depends on, never an address.
-constexpr size_t kMaxSearchedPlans = 256;
+// kept by structure: everything the plan depends on, never an address.  At most
+// 32 MiB of them (about 28 bytes per op), all given back at once when full.
+constexpr size_t kMaxSearchedBytes = 32u << 20;
 std::mutex g_search_mu;
+size_t g_searched_bytes = 0;
 std::unordered_map<std::string, std::vector<Segment>> g_searched;
 }  // namespace
 
@@ -259,9 +261,15 @@ int plan_segments(int n, const std::vector<KOp>& ops, const PlanCfg& pc, std::ve
     LQS_TRY(make_plan(n, po, pc, true, alt));
     if (alt.size() < segs.size()) segs.swap(alt);
   }
+  size_t bytes = key.size() + 64;
+  for (const Segment& s : segs) bytes += sizeof s + s.ops.size() * sizeof s.ops[0];
+  if (bytes > kMaxSearchedBytes) return LQS_OK;
   std::lock_guard<std::mutex> lk(g_search_mu);
-  if (g_searched.size() >= kMaxSearchedPlans) g_searched.clear();
-  g_searched.emplace(std::move(key), segs);
+  if (g_searched_bytes + bytes > kMaxSearchedBytes) {
+    g_searched.clear();
+    g_searched_bytes = 0;
+  }
+  if (g_searched.emplace(std::move(key), segs).second) g_searched_bytes += bytes;
   return LQS_OK;
 }
 

@@ -5,7 +5,9 @@ ops segment by segment (original relative order inside a segment) through the
 CPU oracle must therefore reproduce the in-order result; and every segment's
 tile must hold the low qubits and every non-diagonal target of its gates.
 """
+import ctypes
 import math
+import os
 import time
 
 import numpy as np
@@ -185,5 +187,28 @@ def test_planning_time_is_proportional_to_the_circuit():
         L.lqs_set_jit(L.LQS_JIT_ON)
         small = min(seconds(4000, s) for s in (1, 2, 3))
         assert seconds(32000, 4) <= 16 * small
+    finally:
+        L.lqs_set_jit(old)
+
+
+def test_kept_plans_are_bounded_in_bytes():
+    """Sixty plans of 100000 ops (2.8 MB each with their keys) leave no more than the store's 32 MiB behind, and as much
+    again for what the allocator keeps."""
+    def resident():
+        ctypes.CDLL(None).malloc_trim(0)  # freed blocks between live ones
+        with open("/proc/self/statm") as f:
+            return int(f.read().split()[1]) * os.sysconf("SC_PAGE_SIZE")
+
+    c = W.Circuit(13)
+    c.ops = [W.Op("X", (i % 12,)) for i in range(100000)]
+    ops = L.OpArray(c.ops)
+    old = L.lqs_jit_info()["mode"]
+    try:
+        L.lqs_set_jit(L.LQS_JIT_ON)
+        L.lqs_plan_fused(13, "c128", ops, {"max_ops": 60})
+        before = resident()
+        for max_ops in range(61, 121):
+            L.lqs_plan_fused(13, "c128", ops, {"max_ops": max_ops})
+        assert resident() - before <= 2 * (32 << 20)
     finally:
         L.lqs_set_jit(old)
