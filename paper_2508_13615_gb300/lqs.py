@@ -302,6 +302,8 @@ def lqs_check_bounded_wait(h) -> None:
 #: small argument arrays, by length (building a ctypes array type costs more than filling one)
 _INTS = [ctypes.c_int * max(k, 1) for k in range(9)]
 _DOUBLES = [ctypes.c_double * max(k, 1) for k in range(9)]
+#: gates that take a matrix in place of angles
+_MATRIX_GATES = (GATE_IDS["U2"], GATE_IDS["U4"])
 
 
 def lqs_apply_gate(h, gate, wires: Sequence[int], params=(), inverse: bool = False) -> None:
@@ -309,13 +311,13 @@ def lqs_apply_gate(h, gate, wires: Sequence[int], params=(), inverse: bool = Fal
     gid = GATE_IDS[gate] if isinstance(gate, str) else int(gate)
     nw = len(wires)
     w = (_INTS[nw] if nw < 9 else ctypes.c_int * nw)(*[int(x) for x in wires])
-    if type(params) in (tuple, list) and len(params) < 9 and gid not in (17, 18) and all(
+    if type(params) in (tuple, list) and len(params) < 9 and gid not in _MATRIX_GATES and all(
             type(x) is float for x in params):
         # a small state's gate takes a few microseconds: plain floats go over without numpy
         npar = len(params)
         _check(_L.lqs_apply_gate(h, gid, w, nw, _DOUBLES[npar](*params), npar, int(bool(inverse))))
         return
-    if gid in (GATE_IDS["U2"], GATE_IDS["U4"]):
+    if gid in _MATRIX_GATES:
         p = np.ascontiguousarray(np.asarray(params, dtype=np.complex128).reshape(-1)).view(np.float64).copy()
         npar = int(p.size)
     else:
