@@ -91,6 +91,14 @@ constexpr int kMaxGradSlotsJit = 128;  // gradient slots per compiled adjoint se
 // qubits kept the error of normalised double-float (2.5e-14) with up to 32
 // updates between renormalisations, and 2-5x that at 64-128.
 constexpr int kRenormEvery = 16;
+// ... and between renormalisations merged diagonal runs, whose factors carry
+// errors of their own.  Searched plans put up to six runs into a pass where
+// program order had two; error against 64 bits of the 24-qubit universal
+// circuit with program order 3.3e-14, searched without this limit 5.5e-14, with
+// limits of 4 / 3 / 2 (and normalised factors, see emit_op K_DPROD) 3.5 / 3.3 /
+// 3.2e-14; it costs 2.1 / 2.6 / 3.3% of that circuit's time and 0.2 / 0.7 / 1.0%
+// of the 30-qubit ansatz's.
+constexpr int kRenormRuns = 3;
 
 // A forward program's unit-row forms leave every amplitude scaled by 1/g, the
 // product of their factors.  The scalar commutes with every op, so it is
@@ -144,6 +152,7 @@ class SegGen {
   int nut_ = 0;   // entries of the shared tables of tile-independent diagonal runs (UT)
   std::vector<std::string> ofac_;  // per run with outside factors: its per-tile product (OF)
   int lz_ = 0;    // amplitude updates since the registers were last renormalised
+  int runs_ = 0;  // merged diagonal runs since then
   // Exchanges since the last block-wide barrier, for the ordering check of
   // a buffer's next writes (exchange_safe): per exchange its buffer, the warp
   // writing and the warp reading each buffer position, and its barrier's
@@ -1121,7 +1130,10 @@ bool SegGen::emit_op(const TOp& t) {
           }
         }
         tab[0] = a;
-        // products for the needed factor patterns, each from a smaller one
+        // products for the needed factor patterns, each from a smaller one;
+        // those that further products start from are normalised (up to four
+        // unnormalised products in a row gave 7.4e-14 against 64 bits in the
+        // 30-qubit ansatz, 6.8e-14 this way)
         std::vector<uint32_t> all;
         for (uint32_t key : need)
           for (uint32_t x = key; x; x &= ~(1u << (31 - __builtin_clz(x)))) all.push_back(x);
@@ -1130,7 +1142,9 @@ bool SegGen::emit_op(const TOp& t) {
         for (uint32_t key : all) {
           const int m = 31 - __builtin_clz(key);
           const std::string nm = fresh("f");
-          o_ << "      const C " << nm << " = lqs::jit::Lz<A>::kmul(" << cref(lidx(slot_[m])) << ", " << tab[key ^ (1u << m)]
+          bool inner = false;
+          for (uint32_t x : all) inner = inner || (x > key && (x & ((2u << m) - 1u)) == key);
+          o_ << "      const C " << nm << " = lqs::jit::Lz<A>::" << (inner ? "kmuln" : "kmul") << "(" << cref(lidx(slot_[m])) << ", " << tab[key ^ (1u << m)]
              << ");\n";
           tab[key] = nm;
         }
@@ -1319,12 +1333,13 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
     const TOp& t = ops[i];
     const bool plain = (t.kind == K_ANTI1 && t.special == 1) || (t.kind == K_PHASE && t.special != 0) ||
                        t.kind == K_SWAP || t.kind == K_GRAD;
-    if (!plain && ++lz_ >= kRenormEvery) {
+    if (t.kind == K_DPROD) ++runs_;
+    if (!plain && (++lz_ >= kRenormEvery || runs_ >= kRenormRuns)) {
       o_ << "    // renormalise the double-float registers\n";
       each([&]() {
         for (int e = 0; e < R_; ++e) o_ << "    lqs::jit::renorm<A>(" << V(e) << ");\n";
       });
-      lz_ = 0;
+      lz_ = runs_ = 0;
     }
   }
   flush_pending(true);

@@ -36,6 +36,7 @@ template <class A> struct Lz {
     return A::rmac2(c0, a, c1, b);
   }
   static __device__ __forceinline__ C kmul(const C& a, const C& b) { return A::kmul(a, b); }
+  static __device__ __forceinline__ C kmuln(const C& a, const C& b) { return A::kmul(a, b); }  // normalised
   static __device__ __forceinline__ void renorm(W&) {}
   // SX x + k y for a real k
   template <int SX>
@@ -132,11 +133,14 @@ template <> struct Lz<ArDFP> {
     for (int i = 1; i < 4; ++i) cmac(A, k2(c[i]), a[i]);
     return p2_raw(A);
   }
-  static __device__ __forceinline__ DFK kmul(const DFK& a, const DFK& b) {
+  static __device__ __forceinline__ DFK lanes(const P2& w) {
     DFK r;
-    p2_lanes(cmul(a, P2{f2_pack(b.re.h, b.im.h), f2_pack(b.re.l, b.im.l)}), r.re, r.im);
+    p2_lanes(w, r.re, r.im);
     return r;
   }
+  static __device__ __forceinline__ P2 pair(const DFK& b) { return P2{f2_pack(b.re.h, b.im.h), f2_pack(b.re.l, b.im.l)}; }
+  static __device__ __forceinline__ DFK kmul(const DFK& a, const DFK& b) { return lanes(p2_raw(cprod(k2(a), pair(b)))); }
+  static __device__ __forceinline__ DFK kmuln(const DFK& a, const DFK& b) { return lanes(p2_norm(cprod(k2(a), pair(b)))); }
   static __device__ __forceinline__ W rmac2(const R2& c0, const W& a, const R2& c1, const W& b) {
     PAcc A = p2_prod(a, P2{c0.h, c0.l});
     p2_mac(A, b, P2{c1.h, c1.l});

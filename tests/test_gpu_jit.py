@@ -368,3 +368,20 @@ def test_universal_circuit_vs_oracle(jit_on, dtype, arith, n):
         with gpu_state(n, dtype, psi0) as sv:
             sv.apply(c, fused=fused)
             check_state(sv.numpy(), want, dtype, len(c.ops), fused)
+
+
+def test_full_segments_keep_the_precision_of_short_ones(jit_on):
+    """A pass that applies many layers' diagonal products rounds no worse than passes of one layer each, which leave
+    normalised amplitudes behind: the error of the universal circuit against float64 may be a quarter above theirs."""
+    L, _ = jit_on
+    set_mode("df")
+    n = 16
+    c = W.universal(n)
+    psi0 = W.gaussian_state(n, 11)
+    want = oracle.run_circuit(c, psi0.copy())
+    err = []
+    for cfg in (None, {"max_ops": 2 * n - 1}):
+        with gpu_state(n, "c128", psi0) as sv:
+            L.lqs_apply_fused(sv.h, L.OpArray(c.ops), c.params, cfg)
+            err.append(float(np.linalg.norm(sv.numpy() - want) / np.linalg.norm(want)))
+    assert err[0] <= 1.25 * err[1], err
