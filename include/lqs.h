@@ -410,11 +410,12 @@ LQS_API int lqs_jit_info(lqs_jit_stats* out);
 LQS_API int lqs_jit_precompile(int n_qubits, int dtype, int arith, const lqs_op* ops, int n_ops,
                                const double* params, int n_params, const lqs_fuse_cfg* cfg, int* n_compiled);
 /* The same for the reverse sweep of lqs_adjoint_grad on this circuit: its compiled kernels hold psi and
- * lambda in registers (tiles one qubit smaller than lqs_apply_fused's, 256 threads) and add each
+ * lambda in registers (tiles of 2^11 amplitudes of each; 256 threads for c128, 512 for c128 with
+ * LQS_ARITH_F64, 128 for c64) and add each
  * parameter's Im<lambda|G|psi> as they un-apply the gates.  lqs_adjoint_grad uses them whenever compiled
  * segments are enabled for the state's size (LQS_JIT_ON, or LQS_JIT_AUTO on 20 or more qubits),
- * compiling missing ones at that call; states of at most 11 (c128) / 12 (c64) qubits use the
- * shared-memory sweep and compile nothing here. */
+ * compiling missing ones at that call; states of at most 11 qubits use the shared-memory sweep and
+ * compile nothing here. */
 LQS_API int lqs_jit_precompile_adjoint(int n_qubits, int dtype, int arith, const lqs_op* ops, int n_ops,
                                        const double* params, int n_params, int* n_compiled);
 /* The same for the expectation-value passes of lqs_expval on these terms (lambda = 0), or for the passes

@@ -248,8 +248,10 @@ __device__ __forceinline__ f2 f2_conj(f2 a) { return a ^ 0x8000000000000000ull; 
 // Two double-floats to a register pair, usually the components of one
 // amplitude: the leading parts of (re, im) and their low parts.  Every
 // operation runs on both components at once, in the order and with the
-// roundings of the scalar forms (arith.cuh df_prod, df_mac), so results are
-// those of ArDF bit for bit.
+// roundings of the scalar forms (arith.cuh df_prod, df_mac), so gate updates
+// are those of the scalar forms bit for bit.  Sums over amplitudes (gradient
+// and Pauli partials) are not: they keep one sum per component and add the two
+// at the end, where the scalar form adds every term to one sum.
 struct P2 { f2 h, l; };   // two double-floats
 struct PAcc { f2 s, e; };  // two accumulators (leading sums, collected errors)
 __device__ __forceinline__ P2 p2_raw(const PAcc& a) { return P2{a.s, a.e}; }

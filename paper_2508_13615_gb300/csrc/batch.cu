@@ -424,7 +424,7 @@ struct QPart {
   std::vector<PWord> words;
   std::vector<double> wcoef;
   std::vector<BGen> gens;
-  int npas = 0, nrev = 0;
+  int npas = 0;  // Pauli stages so far
   double cost = 0.0;
   int rc = LQS_OK;
   std::string err;
@@ -500,9 +500,7 @@ static int build_part(const lqs_batch_item& it, int dtype, int index, QPart<A>& 
     Q.stages.push_back(st);
     ++Q.npas;
   }
-  const size_t r0 = Q.stages.size();
   LQS_TRY(append_segs(Q, n, sh, rev, plan->rev, QS_REV));
-  Q.nrev = (int)(Q.stages.size() - r0);
   if (!Q.stages.empty()) Q.stages[0].init = 1;
   Q.cost = std::ldexp((double)Q.stages.size() + 1.0, n);
   return LQS_OK;
@@ -701,7 +699,7 @@ static int batch_run_t(const lqs_batch_item* items, int n_items, int dtype, cuda
   a.kmax = kmax;
   a.first = reinterpret_cast<const int*>(d + o_fs);
   a.sums = outs;
-  // 4. the task kernel on every SM, then the per-circuit reduction
+  // 4. the task kernel on every SM, then the reduction of every stage's partial sums
   const size_t smem = 2 * ((size_t)sizeof(typename A::W) << kmax) + sizeof(double) * kTileWarps * kMaxGradSlots;
   static std::once_flag attr_once;
   cudaError_t ae = cudaSuccess;

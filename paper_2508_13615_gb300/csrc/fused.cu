@@ -162,7 +162,7 @@ int fill_segment(const std::vector<POp>& ops, const std::vector<int>& rem, size_
 // with a CNOT ladder advance in skewed windows this way (half the qubits per
 // layer, two to five layers per pass): 30-qubit 10-layer ansatz, complex128 33
 // -> 27 passes (21 with a dense cap of 16) and 444 -> 418 ms; 24-qubit
-// universal circuit 55 -> 23 and 6.29 -> 5.29 ms.  Tiles are weighed on the ops
+// universal circuit 55 -> 23 and 6.29 -> 5.43 ms.  Tiles are weighed on the ops
 // just ahead (1024: eleven layers of 30 qubits), so that the time of the search
 // is proportional to the circuit's length.  The scan ends early only where every
 // wire is blocked, and one that is only a control never is: 16000 ops on 30

@@ -1162,11 +1162,14 @@ bool SegGen::emit_op(const TOp& t) {
   }
 }
 
-// Kernels run two CTAs per SM, each with one buffer per tile: bulk loads land in it, and once the tile is in registers the layout exchanges go
-// through it.  After the last exchange has been read the buffer is free and
-// the next tile's load starts, behind the remaining ops and the stores of this
-// tile and the whole work of the other CTA.  FP32 pipe busy 57-68% against
-// 52-56% with one CTA per SM and a prefetch buffer (24-qubit ansatz).
+// Kernels share an SM (two CTAs; four in the complex64 reverse sweep; one of
+// 512 threads in the float64 policy), each with one buffer per tile: bulk loads
+// land in it, and once the tile is in registers the layout exchanges go through
+// it.  After the last exchange has been read the buffer is free and the next
+// tile's load starts, behind the remaining ops and the stores of this tile and
+// the whole work of the other CTAs.  With one CTA per SM and a prefetch buffer
+// the FP32 pipe was busy 52-56% of the time; now: the segment profile under
+// profiles/.
 const char* kSkeletonHead = R"(
 extern "C" __global__ void __launch_bounds__(@NTH@, @MINB@)
 @NAME@(A::S* __restrict__ psi, @LAMP@const __grid_constant__ SegArgs P, @PARTP@int* status@FMTP@) {
@@ -1401,7 +1404,9 @@ bool SegGen::run(const TOp* ops, int nops, int ncoef, int ngrad, std::string& sr
   // resident CTAs per SM the register budget aims at: two (1024 threads per SM
   // with 128 bytes of states per thread, 512 with 256), one for 512 threads of
   // float64 (64 registers spill, and its pipe is busy anyway; 24 qubits, one
-  // against two: U4 windows 32.6 and 33.7 ms, RX + RZ 28.7 and 29.5)
+  // against two: U4 windows 32.6 and 33.7 ms, RX + RZ 28.7 and 29.5).  Long
+  // complex64 segments spill up to 780 bytes at two and are faster all the same:
+  // 7-layer ansatz on 28 qubits 19.7 against 27.5 ms, U4 windows 8.7 against 9.5
   const bool f64 = aname_ == std::string("lqs::ArF64");
   const int minb = f64 && nth >= 512 ? 1 : std::max(1, (R_ * sz_ * (adj_ ? 2 : 1) <= 128 ? 1024 : 512) / nth);
   head = replace_all(head, "@MINB@", std::to_string(minb));
